@@ -10,6 +10,7 @@
 #include "hh_internal.h"
 #include "hh_cycle.h"
 #include "hh_gmres.h"
+#include "hh_gmres2d.h"
 #include "hh_krylov.h"
 #include "hh_tiled3d.h"
 
@@ -95,6 +96,8 @@ struct LevelHost {
   int ulo[2] = {1, 1}, uhi[2] = {0, 0};  // uniform-coefficient node range per dir
   double2 c0_64[2];
   float2 c0_32[2];
+  double2 sig64[2];    // GMRES smoothing: centre of the level's spectrum and
+  double gs = 0.0;     // inverse half width (hh_cheb.cuh)
 };
 
 struct GraphEntry {
@@ -139,9 +142,12 @@ struct hh_handle {
   CoarseGroup groups[MAXL];
   int parts_cap = 0;                // capacity of `partials` per RHS
   int gm_cap = 0;                   // most blocks of a GMRES smoothing kernel
-  int gm_fuse = 1;                  // fused orthogonalisation + Arnoldi kernels
-  int gm_col = 1;                   // ... marching down columns on large 2-D levels
-  int gm_col_min = 256;             // (from this many points per axis)
+  int gm_fuse = 1;                  // 3-D: fused orthogonalisation + Arnoldi kernels
+  int sms = 0;                      // SMs of the device
+  void *gm2_parts = nullptr;        // 2-D: partial Gram matrices of a step,
+  int *gm2_zero = nullptr;          // whether it started from zero (per right-hand side),
+  double *gm2_coef = nullptr;       // complex128: coefficients and their correction's sums
+  double *gm2_parts2 = nullptr;
   int pw3d = 0;                     // 3-D: point-wise kernels instead of the tile-staged ones
   cudaStream_t side = nullptr;      // branch of the stop test in the fused cycle
   cudaStream_t grp = nullptr;       // this handle's stream in a group solve (lazy)
@@ -348,19 +354,114 @@ int partial_blocks_of(const hh_handle *h, int l) {
   return l == 0 ? h->nparts : gmres_blocks(h, l);
 }
 
-// Kernel options of a GMRES smoothing step on a level of N points per axis
-// (launch_gmres_rest's fuse bits): fused orthogonalisation + Arnoldi, and on
-// 2-D levels with N >= gm_col_min the column-marching kernels.
-int gm_flags(const hh_handle *h, int N) {
-  return h->gm_fuse | ((h->gm_col && h->dim == 2 && N >= h->gm_col_min) ? 2 : 0);
+int tune_batch(const hh_handle *h);
+void fork_check(hh_handle *h, int check, unsigned long long cond, cudaStream_t s);
+
+// 2-D GMRES steps (hh_gmres2d.h): constants of a level, workspace and split.
+template <typename R> struct Gm2dLevel {
+  LevelK<R> K;
+  typename Cx<R>::T sigma;
+  R s;
+  Gm2dWork<R> w;
+};
+template <typename R> Gm2dLevel<R> gm2d_level(hh_handle *h, int l, int dir) {
+  const LevelHost &v = h->lv[l];
+  Gm2dLevel<R> g;
+  g.K = levelk<R>(h, l, dir);
+  g.sigma.x = (R)v.sig64[dir].x;
+  g.sigma.y = (R)v.sig64[dir].y;
+  g.s = (R)v.gs;
+  g.w.parts = reinterpret_cast<typename GramSum<R>::T *>(h->gm2_parts);
+  g.w.zflag = h->gm2_zero;
+  g.w.q = work<R>(h).gq[l];
+  g.w.qs = (size_t)v.S * h->max_batch;
+  g.w.coef = h->gm2_coef;
+  g.w.parts2 = h->gm2_parts2;
+  return g;
+}
+// The split is that of the handle's batch capacity (at most 16), so that the
+// stop test's number of partial sums does not depend on the call.
+template <typename R> Gm2dPlan gm2d_plan_of(const hh_handle *h, int l, bool restrict_) {
+  return gm2d_plan<R>(h->lv[l].N, h->opt.gmres_m, tune_batch(h), h->sms, restrict_);
 }
 
-// The V-cycle with GMRES(m) smoothing (Sec. 3.2): on each level nu1 GMRES
+// One GMRES step on level l (2-D): u_out = in + z; with fc the restricted
+// residual of u_out as well.
+template <typename R>
+void enqueue_gm2d_step(hh_handle *h, int l, int dir, const Gm2dIn<R> &in, typename Cx<R>::T *u_out,
+                       bool restrict_, int batch, const SolveState *st, int check,
+                       unsigned long long cond, cudaStream_t s) {
+  const Gm2dLevel<R> g = gm2d_level<R>(h, l, dir);
+  const Gm2dPlan p = gm2d_plan_of<R>(h, l, restrict_);
+  const int m = h->opt.gmres_m;
+  launch_gm2d_basis<R>(g.K, g.sigma, g.s, h->kconst, m, in, g.w, p, batch, st,
+                       stop_test(check) ? h->partials : nullptr, s);
+  if (stop_test(check)) fork_check(h, check, cond, s);
+  launch_gm2d_update<R>(g.K, g.sigma, g.s, h->kconst, m, in, g.w, p, u_out,
+                        restrict_ ? work<R>(h).f[l + 1] : nullptr, cscal<R>(h, l, dir),
+                        restrict_ ? lay_of(h, l + 1) : Lay{0, 0, 0}, batch, st, s);
+}
+
+template <typename R>
+void enqueue_gmres_tail(hh_handle *h, int dir, int batch, const SolveState *st, cudaStream_t s) {
+  auto go = [&](auto &a) {
+    if (h->dim == 2) launch_gmres_tail<R, 2>(a, batch, st, s);
+    else launch_gmres_tail<R, 3>(a, batch, st, s);
+  };
+  if constexpr (std::is_same<R, float>::value) go(h->gta32[dir]);
+  else go(h->gta64[dir]);
+}
+
+// The 2-D V-cycle with GMRES(m) smoothing: two kernels per step; the last
+// pre-smoothing step restricts its residual, the first post-smoothing step
+// starts from the corrected iterate.  On level 0 the first step's |f - A u|^2
+// is the stop test's, which runs on a branch beside the coarser levels and is
+// joined before the one part of the cycle that writes the level-0 iterate (the
+// level-0 post-smoothing; see fork_check).
+template <typename R>
+void enqueue_cycle_gmres2d(hh_handle *h, int dir, int batch, int zero0, int check,
+                           unsigned long long cond, cudaStream_t s) {
+  using C = typename Cx<R>::T;
+  Work<R> &W = work<R>(h);
+  const SolveState *st = check != CHECK_NONE ? h->st : nullptr;
+  const int L = h->L, T = h->gtail0 > 0 ? h->gtail0 : L - 1;
+  const int nu1 = h->opt.nu1, nu2 = h->opt.nu2;
+  for (int l = 0; l < T; ++l) {
+    const C *in = l == 0 ? W.u_post[0] : W.u_pre[l];
+    int zm = l == 0 ? zero0 : ZERO_ALL;
+    for (int j = 0; j < nu1; ++j) {
+      C *out = (nu1 - 1 - j) % 2 == 0 ? W.u_pre[l] : W.tmp[l];
+      const Gm2dIn<R> a{in, W.f[l], nullptr, Lay{0, 0, 0}, zm};
+      enqueue_gm2d_step<R>(h, l, dir, a, out, j == nu1 - 1, batch, st,
+                           l == 0 && j == 0 ? check : CHECK_NONE, cond, s);
+      in = out;
+      zm = ZERO_NONE;
+    }
+  }
+  if (h->gtail0 > 0)
+    enqueue_gmres_tail<R>(h, dir, batch, st, s);
+  else
+    launch_coarse_solve<R, 2>(h->lu[dir], h->piv[dir], lay_of(h, L - 1), W.f[L - 1],
+                              W.u_post[L - 1], batch, st, s);
+  for (int l = T - 1; l >= 0; --l) {
+    if (l == 0 && stop_test(check)) cudaStreamWaitEvent(s, h->ev_join, 0);
+    const C *in = W.u_pre[l];
+    for (int j = 0; j < nu2; ++j) {
+      C *out = (nu2 - 1 - j) % 2 == 0 ? W.u_post[l] : W.tmp[l];
+      const Gm2dIn<R> a{in, W.f[l], j == 0 ? W.u_post[l + 1] : nullptr, lay_of(h, l + 1), ZERO_NONE};
+      enqueue_gm2d_step<R>(h, l, dir, a, out, false, batch, st, CHECK_NONE, cond, s);
+      in = out;
+    }
+  }
+}
+
+// The 3-D V-cycle with GMRES(m) smoothing (Sec. 3.2): on each level nu1 GMRES
 // steps, residual + restriction, recursion, correction, nu2 GMRES steps.
 // On level 0 the first step's residual is the stop test's.
-template <typename R, int DIM>
-void enqueue_cycle_gmres(hh_handle *h, int dir, int batch, int zero0, int check,
+template <typename R>
+void enqueue_cycle_gmres3d(hh_handle *h, int dir, int batch, int zero0, int check,
                          unsigned long long cond, cudaStream_t s) {
+  constexpr int DIM = 3;
   Work<R> &W = work<R>(h);
   const SolveState *st = check != CHECK_NONE ? h->st : nullptr;
   const int L = h->L, m = h->opt.gmres_m;
@@ -374,19 +475,18 @@ void enqueue_cycle_gmres(hh_handle *h, int dir, int batch, int zero0, int check,
     int zm = l == 0 ? zero0 : ZERO_ALL;
     for (int j = 0; j < h->opt.nu1; ++j) {
       const bool norm = l == 0 && j == 0 && stop_test(check);
-      launch_gmres_start<R, DIM>(K, in, zm, W.f[l], g, batch, st, norm ? h->partials : g.parts, nb, s,
-                                 gm_flags(h, K.N) & 2);
+      launch_gmres_start<R, DIM>(K, in, zm, W.f[l], g, batch, st, norm ? h->partials : g.parts, nb, s);
       if (norm) {
         if (check == CHECK_CYCLE)
           launch_check_cycle(h->st, h->partials, h->params, h->flag, cond, h->copies, h->err, s);
         else
           launch_check_inner(h->st, h->partials, h->params, h->flag, cond, h->copies, h->err, s);
       }
-      launch_gmres_rest<R, DIM>(K, in, zm, W.u_pre[l], g, m, batch, st, nb, s, gm_flags(h, K.N));
+      launch_gmres_rest<R, DIM>(K, in, zm, W.u_pre[l], g, m, batch, st, nb, s, h->gm_fuse);
       in = W.u_pre[l];
       zm = ZERO_NONE;
     }
-    if (DIM == 3 && !pointwise3d(h))
+    if (!pointwise3d(h))
       launch_resid_restrict3d<R>(K, W.u_pre[l], W.f[l], W.f[l + 1], lay_of(h, l + 1),
                                  cscal<R>(h, l, dir), batch, st, s);
     else
@@ -394,10 +494,7 @@ void enqueue_cycle_gmres(hh_handle *h, int dir, int batch, int zero0, int check,
                                     cscal<R>(h, l, dir), batch, st, s);
   }
   if (h->gtail0 > 0) {
-    if constexpr (std::is_same<R, float>::value)
-      launch_gmres_tail<float, DIM>(h->gta32[dir], batch, st, s);
-    else
-      launch_gmres_tail<double, DIM>(h->gta64[dir], batch, st, s);
+    enqueue_gmres_tail<R>(h, dir, batch, st, s);
   } else {
     launch_coarse_solve<R, DIM>(h->lu[dir], h->piv[dir], lay_of(h, L - 1), W.f[L - 1],
                                 W.u_post[L - 1], batch, st, s);
@@ -409,9 +506,8 @@ void enqueue_cycle_gmres(hh_handle *h, int dir, int batch, int zero0, int check,
     launch_gmres_correct<R, DIM>(K, W.u_pre[l], W.u_post[l + 1], lay_of(h, l + 1), W.u_post[l],
                                  batch, st, s);
     for (int j = 0; j < h->opt.nu2; ++j) {
-      launch_gmres_start<R, DIM>(K, W.u_post[l], ZERO_NONE, W.f[l], g, batch, st, g.parts, nb, s,
-                                 gm_flags(h, K.N) & 2);
-      launch_gmres_rest<R, DIM>(K, W.u_post[l], ZERO_NONE, W.u_post[l], g, m, batch, st, nb, s, gm_flags(h, K.N));
+      launch_gmres_start<R, DIM>(K, W.u_post[l], ZERO_NONE, W.f[l], g, batch, st, g.parts, nb, s);
+      launch_gmres_rest<R, DIM>(K, W.u_post[l], ZERO_NONE, W.u_post[l], g, m, batch, st, nb, s, h->gm_fuse);
     }
   }
 }
@@ -420,7 +516,8 @@ template <typename R, int DIM>
 void enqueue_cycle(hh_handle *h, int dir, int batch, int zero0, int check,
                    unsigned long long cond, cudaStream_t s) {
   if (h->opt.smoother == HH_SMOOTH_GMRES) {
-    enqueue_cycle_gmres<R, DIM>(h, dir, batch, zero0, check, cond, s);
+    if constexpr (DIM == 2) enqueue_cycle_gmres2d<R>(h, dir, batch, zero0, check, cond, s);
+    else enqueue_cycle_gmres3d<R>(h, dir, batch, zero0, check, cond, s);
     return;
   }
   Work<R> &W = work<R>(h);
@@ -999,27 +1096,20 @@ void time_one(hh_handle *h, int kernel, int level, int batch, cudaStream_t s) {
   const auto om = omega<R>(h, 0);
   const bool two = h->dim == 2;
   if (kernel == 6) {   // one GMRES(m) smoothing step from a nonzero iterate
-    const GmresWork<R> g = gmres_work<R>(h, level);
-    const int nb = partial_blocks_of(h, level), m = h->opt.gmres_m;
-    typename Cx<R>::T *u = W.u_post[level];
     if (two) {
-      launch_gmres_start<R, 2>(K, u, ZERO_NONE, W.f[level], g, batch, nullptr, g.parts, nb, s,
-                               gm_flags(h, K.N) & 2);
-      launch_gmres_rest<R, 2>(K, u, ZERO_NONE, u, g, m, batch, nullptr, nb, s, gm_flags(h, K.N));
+      const Gm2dIn<R> in{W.u_post[level], W.f[level], nullptr, Lay{0, 0, 0}, ZERO_NONE};
+      enqueue_gm2d_step<R>(h, level, 0, in, W.u_pre[level], false, batch, nullptr, CHECK_NONE, 0, s);
     } else {
+      const GmresWork<R> g = gmres_work<R>(h, level);
+      const int nb = partial_blocks_of(h, level), m = h->opt.gmres_m;
+      typename Cx<R>::T *u = W.u_post[level];
       launch_gmres_start<R, 3>(K, u, ZERO_NONE, W.f[level], g, batch, nullptr, g.parts, nb, s);
-      launch_gmres_rest<R, 3>(K, u, ZERO_NONE, u, g, m, batch, nullptr, nb, s, gm_flags(h, K.N));
+      launch_gmres_rest<R, 3>(K, u, ZERO_NONE, u, g, m, batch, nullptr, nb, s, h->gm_fuse);
     }
     return;
   }
   if (kernel == 4 && h->opt.smoother == HH_SMOOTH_GMRES) {   // the GMRES one-block tail
-    if constexpr (std::is_same<R, float>::value) {
-      if (two) launch_gmres_tail<float, 2>(h->gta32[0], batch, nullptr, s);
-      else launch_gmres_tail<float, 3>(h->gta32[0], batch, nullptr, s);
-    } else {
-      if (two) launch_gmres_tail<double, 2>(h->gta64[0], batch, nullptr, s);
-      else launch_gmres_tail<double, 3>(h->gta64[0], batch, nullptr, s);
-    }
+    enqueue_gmres_tail<R>(h, 0, batch, nullptr, s);
     return;
   }
   if (kernel == 4) {
@@ -1698,6 +1788,14 @@ hh_status autotune(hh_handle *h, cudaStream_t s) {
 // GMRES smoothing: the one-block tail runs the levels from the first one
 // whose tail (it and all coarser levels) fits kGmTailSmemMax of shared
 // memory (HH_GMTAIL=off in the environment keeps every level per-level).
+// Largest level (points per axis) of the GMRES one-block tail (HH_GMTAIL_N
+// overrides, for tuning).
+template <typename R> int gm_tail_max_n(int dim) {
+  if (const char *e = std::getenv("HH_GMTAIL_N")) return std::max(3, std::atoi(e));
+  if (dim == 3) return 15;
+  return sizeof(R) == 4 ? 31 : 15;
+}
+
 template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
   h->gtail0 = 0;
   const char *ge = std::getenv("HH_GMTAIL");
@@ -1710,6 +1808,7 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
     for (int l = t; l < L; ++l) N[l - t] = h->lv[l].N;
     const size_t b = h->dim == 2 ? gmres_tail_smem<R, 2>(N, L - t, h->opt.gmres_m)
                                  : gmres_tail_smem<R, 3>(N, L - t, h->opt.gmres_m);
+    if (N[0] > gm_tail_max_n<R>(h->dim)) continue;
     if (b <= kGmTailSmemMax) { t0 = t; break; }
   }
   if (t0 < 0) return HH_OK;
@@ -1721,7 +1820,7 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
     a.m = h->opt.gmres_m;
     a.nu1 = h->opt.nu1;
     a.nu2 = h->opt.nu2;
-    auto pts = [&](int n) { return h->dim == 2 ? (size_t)n * n : (size_t)n * n * n; };
+    auto pts = [&](int n) { return (size_t)(n + 1) * (h->dim == 2 ? n : n * n); };   // pitched
     size_t c = 0, r = 0;
     for (int q = 0; q < 3; ++q) { a.offQ[q] = (int)c; c += pts(h->lv[t0].N); }
     for (int i = 0; i < a.nl; ++i) {
@@ -1729,6 +1828,9 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
       GmTailLevel<R> &g = a.lv[i];
       g.K = levelk<R>(h, l, dir);
       g.c = cscal<R>(h, l, dir);
+      g.sigma.x = (R)h->lv[l].sig64[dir].x;
+      g.sigma.y = (R)h->lv[l].sig64[dir].y;
+      g.s = (R)h->lv[l].gs;
       g.offU = (int)c; c += pts(h->lv[l].N);
       g.offF = (int)c; c += pts(h->lv[l].N);
       g.offT = (int)c; c += 3 * (size_t)h->dim * h->lv[l].N;
@@ -1909,18 +2011,20 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   h->k2c = k2_dev ? 0.0 : k2_const;
   h->fused = 0;
   if (h->opt.smoother == HH_SMOOTH_GMRES) {
-    // Krylov vectors per level (cycle precision), partial sums for up to six
-    // quantities per block, the arrival counter and the per-RHS scalars
+    // vectors per level, in the cycle's precision: 3-D q_0..q_3 and two of
+    // A q_j; 2-D complex128 q_0..q_2 and X q_2 (complex64 stores none)
     for (int l = 0; l + 1 < L; ++l) {
       const size_t np = (size_t)h->lv[l].S * B;
       if (h->opt.precision == HH_FP64) {
         HH_TRY(dev_alloc_n(h, &h->w64.gq[l], 4 * np));
-        HH_TRY(dev_alloc_n(h, &h->w64.gw[l], np));
-        HH_TRY(dev_alloc_n(h, &h->w64.gw2[l], np));
         HH_CK(cudaMemsetAsync(h->w64.gq[l], 0, 4 * np * sizeof(double2), s));
-        HH_CK(cudaMemsetAsync(h->w64.gw[l], 0, np * sizeof(double2), s));
-        HH_CK(cudaMemsetAsync(h->w64.gw2[l], 0, np * sizeof(double2), s));
-      } else {
+        if (dim == 3) {
+          HH_TRY(dev_alloc_n(h, &h->w64.gw[l], np));
+          HH_TRY(dev_alloc_n(h, &h->w64.gw2[l], np));
+          HH_CK(cudaMemsetAsync(h->w64.gw[l], 0, np * sizeof(double2), s));
+          HH_CK(cudaMemsetAsync(h->w64.gw2[l], 0, np * sizeof(double2), s));
+        }
+      } else if (dim == 3) {
         HH_TRY(dev_alloc_n(h, &h->w32.gq[l], 4 * np));
         HH_TRY(dev_alloc_n(h, &h->w32.gw[l], np));
         HH_TRY(dev_alloc_n(h, &h->w32.gw2[l], np));
@@ -1933,9 +2037,8 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     // stencil loads of the grid-stride loops in flight; complex128 2 per SM
     // (bound by the FP64 pipe, where more blocks only lengthen the last
     // block's sum over the partials); HH_GMBLOCKS overrides, for tuning
-    int sms = 0;
-    HH_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    h->gm_cap = (h->opt.precision == HH_FP64 ? 2 : 4) * sms;
+    HH_CK(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device));
+    h->gm_cap = (h->opt.precision == HH_FP64 ? 2 : 4) * h->sms;
     if (const char *e = std::getenv("HH_GMBLOCKS")) h->gm_cap = std::max(1, std::atoi(e));
     HH_TRY(dev_alloc_n(h, &h->gm_parts, (size_t)h->gm_cap * kGmresParts * B));
     // complex64: the orthogonalisation of a step and the next Arnoldi product
@@ -1944,8 +2047,18 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     // bound of those kernels); HH_GMFUSE=0/1 in the environment overrides
     h->gm_fuse = h->opt.precision != HH_FP64;
     if (const char *e = std::getenv("HH_GMFUSE")) h->gm_fuse = std::atoi(e) != 0;
-    if (const char *e = std::getenv("HH_GMCOL")) h->gm_col = std::atoi(e) != 0;
-    if (const char *e = std::getenv("HH_GMCOL_MIN_N")) h->gm_col_min = std::max(1, std::atoi(e));
+    if (dim == 2) {
+      double *q = nullptr;   // 16 sums per block: FP64, or FP32 pairs
+      HH_TRY(dev_alloc_n(h, &q, (size_t)16 * gm2d_max_parts(tune_batch(h), h->sms) * B));
+      h->gm2_parts = q;
+      HH_TRY(dev_alloc_n(h, &h->gm2_zero, (size_t)B));
+      HH_CK(cudaMemsetAsync(h->gm2_zero, 0, (size_t)B * sizeof(int), s));
+      if (h->opt.precision == HH_FP64) {
+        HH_TRY(dev_alloc_n(h, &h->gm2_coef, (size_t)kGm2dCoef * B));
+        HH_TRY(dev_alloc_n(h, &h->gm2_parts2, (size_t)kGm2dCorr * 8 * B));
+      }
+      HH_CK(h->opt.precision == HH_FP64 ? init_gm2d<double>() : init_gm2d<float>());
+    }
     HH_TRY(dev_alloc_n(h, &h->gm_counter, 1));
     HH_CK(cudaMemsetAsync(h->gm_counter, 0, sizeof(unsigned int), s));
     HH_TRY(dev_alloc_n(h, &h->gm_gsc, (size_t)kGmresScalars * B));
@@ -1989,7 +2102,8 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   for (int v = 0; v < kLevel0Variants; ++v)
     h->parts_cap = std::max(h->parts_cap, tile_parts(v, h->lv[0].N));
   if (dim == 3) h->parts_cap = std::max(h->parts_cap, tiles3d(h->lv[0].N));
-  if (h->gm_cap) h->parts_cap = std::max(h->parts_cap, gmres_blocks(h, 0));
+  if (h->gm_cap)
+    h->parts_cap = std::max(h->parts_cap, std::max(gmres_blocks(h, 0), gm2d_max_parts(tune_batch(h), h->sms)));
   HH_TRY(dev_alloc_n(h, &h->partials, (size_t)h->parts_cap * B));
   HH_TRY(dev_alloc_n(h, &h->err, 1));
   HH_CK(cudaMemsetAsync(h->err, 0, sizeof(int), s));
@@ -2005,6 +2119,14 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   if (h->m > 27) return fail(HH_ERR_ARG, "coarsest level too large");
   int *info_d = nullptr;
   HH_TRY(dev_alloc_n(h, &info_d, 2));
+  double *krange_d = nullptr, krange[2] = {k2_const, k2_const};
+  const bool range = h->opt.smoother == HH_SMOOTH_GMRES && k2_dev;
+  if (range) {
+    HH_TRY(dev_alloc_n(h, &krange_d, 2));
+    const LevelHost &v = h->lv[0];
+    launch_k2_range(v.k2_64, v.N, v.P, rows_of(h, 0), krange_d, s);
+    HH_CK(cudaMemcpyAsync(krange, krange_d, sizeof(krange), cudaMemcpyDeviceToHost, s));
+  }
   for (int dir = 0; dir < 2; ++dir) {
     HH_TRY(dev_alloc_n(h, &h->lu[dir], (size_t)h->m * h->m));
     HH_TRY(dev_alloc_n(h, &h->piv[dir], (size_t)h->m));
@@ -2018,6 +2140,17 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   HH_CK(cudaGetLastError());
   if (info_h[0] || info_h[1]) return fail(HH_ERR_ARG, "singular coarsest-level operator");
   if (h->opt.smoother == HH_SMOOTH_GMRES) {
+    // spectrum of a level: 2 dim c_0 - beta k^2 plus the neighbours' part,
+    // |2 dim c_0| at most (coarse k^2 is injected from the fine field)
+    const double kmid = 0.5 * (krange[0] + krange[1]), krad = 0.5 * (krange[1] - krange[0]);
+    for (LevelHost &v : h->lv) {
+      for (int d = 0; d < 2; ++d) {
+        v.sig64[d].x = 2.0 * dim * v.c0_64[d].x - v.beta64[d].x * kmid;
+        v.sig64[d].y = 2.0 * dim * v.c0_64[d].y - v.beta64[d].y * kmid;
+      }
+      v.gs = 1.0 / (2.0 * dim * std::hypot(v.c0_64[0].x, v.c0_64[0].y) +
+                    std::hypot(v.beta64[0].x, v.beta64[0].y) * krad);
+    }
     if (h->opt.precision == HH_MIXED) HH_TRY(setup_gmres_tail<float>(h));
     else HH_TRY(setup_gmres_tail<double>(h));
   }
@@ -2037,7 +2170,10 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   if (dim == 3 && h->opt.smoother == HH_SMOOTH_JACOBI && !pointwise3d(h))
     h->nparts = tiles3d(h->lv[0].N);
   // the GMRES cycle's level-0 start kernel writes one partial sum per block
-  if (h->opt.smoother == HH_SMOOTH_GMRES) h->nparts = gmres_blocks(h, 0);
+  if (h->opt.smoother == HH_SMOOTH_GMRES)
+    h->nparts = dim == 3 ? gmres_blocks(h, 0)
+                         : (h->opt.precision == HH_FP64 ? gm2d_plan_of<double>(h, 0, true)
+                                                        : gm2d_plan_of<float>(h, 0, true)).blocks;
   return HH_OK;
 }
 
@@ -2611,11 +2747,15 @@ int hh_cycle_kernels(const hh_handle *h) {
     if (h->mid && h->opt.precision == HH_MIXED) return 2 * h->mid0 + 2;
     return 2 * (1 + h->ngroups) + 2;
   }
-  if (h->opt.smoother == HH_SMOOTH_GMRES) {  // per level: steps of 2m + 1 kernels
+  if (h->opt.smoother == HH_SMOOTH_GMRES) {
+    // 2-D: two kernels per step (complex128 three); 3-D: per level steps of 2m + 1 kernels
     // (start, m Arnoldi products, m - 1 orthogonalisations, update; m + 2 with
     // the fused orthogonalisation + Arnoldi kernels, m >= 2), residual +
     // restriction, correction; then the tail (or the coarsest LU) and the
     // stop test
+    if (h->dim == 2)
+      return (h->gtail0 > 0 ? h->gtail0 : h->L - 1) * (h->opt.precision == HH_FP64 ? 3 : 2) *
+                 (h->opt.nu1 + h->opt.nu2) + 2;
     const int T = h->gtail0 > 0 ? h->gtail0 : h->L - 1;
     const int m = h->opt.gmres_m;
     const int step = h->gm_fuse && m >= 2 ? m + 2 : 2 * m + 1;

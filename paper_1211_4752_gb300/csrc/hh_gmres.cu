@@ -1,5 +1,7 @@
 // GMRES(m) smoothing (Sec. 3.2, the smoother of the paper's experiments),
-// m <= 3, for every level, 2-D and 3-D, complex64 and complex128.
+// m <= 3, complex64 and complex128: the 3-D levels' kernels and, in 2-D and 3-D,
+// the one-block kernel of the small levels (k_gm_tail, whose steps are those of
+// hh_cheb.cuh).  The other 2-D levels: hh_gmres2d.h.
 //
 // One smoothing step replaces u by u + z, where z minimises ||f - A (u + z)||
 // over the Krylov space K_m(A, r0), r0 = f - A u.  The basis is built without
@@ -24,6 +26,7 @@
 // count.
 #include "hh_kernels.cuh"
 #include "hh_launch.cuh"
+#include "hh_tma.cuh"
 #include "hh_gmres.h"
 
 namespace hh {
@@ -485,235 +488,6 @@ k_gm_orth_arnoldi(LevelK<R> L, typename Cx<R>::T *__restrict__ Q, size_t qs,
                         });
 }
 
-// ---------------------------------------------------------------------------
-// Column-marching versions of Arnoldi step 0 and of the fused
-// orthogonalisation + Arnoldi steps, for large 2-D levels.  A thread owns one
-// column x of a 256-column chunk and marches down a run of rows: the vector
-// the operator is applied to (q_0, or q_{J+1} = w - sum c_iJ q_i) is formed
-// once per point, one row ahead, and kept in registers for the rows above and
-// below; the west and east neighbours come from the adjacent lanes by warp
-// shuffles (a warp's first and last lane form theirs from memory).  Each
-// input vector is read once per point instead of at five stencil points, and
-// q_{J+1} is formed once per point instead of five times.  The per-point
-// arithmetic is the point-wise kernels' (stencil_vals2 adds the neighbour
-// terms in the order of stencil<R, 2>), so iterates agree to rounding of the
-// sums' order.
-// ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ typename Cx<R>::T stencil_vals2(const LevelK<R> &L, int x, int y,
-                                                           typename Cx<R>::T uc,
-                                                           typename Cx<R>::T uw,
-                                                           typename Cx<R>::T ue,
-                                                           typename Cx<R>::T us,
-                                                           typename Cx<R>::T un) {
-  using C = typename Cx<R>::T;
-  const int N = L.N;
-  const C *c = L.coef;
-  C nb = czero<C>();
-  if (x > 0) nb = cfma(c[x], uw, nb);
-  if (x < N - 1) nb = cfma(c[2 * N + x], ue, nb);
-  c += 3 * N;
-  if (y > 0) nb = cfma(c[y], us, nb);
-  if (y < N - 1) nb = cfma(c[2 * N + y], un, nb);
-  const C D = diag_at<R, 2>(L, x, y, 0);
-  return csub(cmul(D, uc), nb);
-}
-
-template <typename C> __device__ __forceinline__ C shfl_c(C v, int delta, bool up) {
-  C r;
-  if (up) {
-    r.x = __shfl_up_sync(0xffffffffu, v.x, delta);
-    r.y = __shfl_up_sync(0xffffffffu, v.y, delta);
-  } else {
-    r.x = __shfl_down_sync(0xffffffffu, v.x, delta);
-    r.y = __shfl_down_sync(0xffffffffu, v.y, delta);
-  }
-  return r;
-}
-
-// OA = false: Arnoldi step 0 (w = A q_0, <q_0, w>), J unused.
-// OA = true: orthogonalise column J and apply the next Arnoldi product (the
-// arithmetic of k_gm_orth_arnoldi<R, 2, J, LAST>; LAST: J + 2 = m).  Grid:
-// nchunk x ceil(N / rows) blocks per right-hand side (blockIdx.x = run *
-// nchunk + chunk).
-template <typename R, bool OA, int J, bool LAST>
-__global__ void __launch_bounds__(256)
-k_gm_col2d(LevelK<R> L, typename Cx<R>::T *__restrict__ Q, size_t qs,
-           const typename Cx<R>::T *__restrict__ w_in, typename Cx<R>::T *__restrict__ w_out,
-           const SolveState *st, double *parts, unsigned int *counter, double *gsc, int nchunk,
-           int rows) {
-  using C = typename Cx<R>::T;
-  static_assert(OA || !LAST, "Arnoldi step 0 of the column kernels is never the last (m >= 2)");
-  constexpr int JJ = OA ? J : -1;        // the last stored column the step reads
-  constexpr int NV = JJ + 1;             // q_0..q_JJ carried for the inner products
-  constexpr int NI = OA ? 1 + 2 * (J + 2) : 2;
-  constexpr int NQ = NI + (LAST ? 1 : 0);
-  static_assert(NQ <= kGmresParts, "partial-sum slots");
-  const int b = blockIdx.y;
-  const bool act = __syncthreads_and(!(st && !st[b].active)) != 0;
-  R acc[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) acc[q] = R(0);
-  R sc[NV > 0 ? NV : 1];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) sc[i] = kscale_of<R>(gsc + b * kGmresScalars, i);
-  const R s_op = kscale_of<R>(gsc + b * kGmresScalars, OA ? J : 0);   // scale of the sums
-  if (act) {
-    const int N = L.N, P = L.P, lane = threadIdx.x & 31;
-    const size_t off = (size_t)b * L.S;
-    const C *qb = Q + off;
-    const C *wb = OA ? w_in + off : nullptr;
-    C c[NV > 0 ? NV : 1];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) c[i] = get_c<R>(gsc + b * kGmresScalars, i, JJ);
-    const int chunk = blockIdx.x % nchunk, run = blockIdx.x / nchunk;
-    const int x = chunk * blockDim.x + threadIdx.x;
-    const int y0 = run * rows, y1 = min(N, y0 + rows);
-    // the inputs of the operand at (xx, yy) (zero outside the domain), and the
-    // operand from them: loading a row two ahead and combining it an iteration
-    // later keeps its loads in flight during the current row's arithmetic
-    struct Raw {
-      C w;
-      C q[NV > 0 ? NV : 1];
-    };
-    auto load = [&](int xx, int yy) {
-      Raw r;
-      r.w = czero<C>();
-#pragma unroll
-      for (int i = 0; i < (NV > 0 ? NV : 1); ++i) r.q[i] = czero<C>();
-      if (xx < 0 || xx >= N || yy < 0 || yy >= N) return r;
-      const size_t o = (size_t)yy * P + xx;
-      if (!OA) {
-        r.w = qb[o];
-        return r;
-      }
-      r.w = wb[o];
-#pragma unroll
-      for (int i = 0; i < NV; ++i) r.q[i] = qb[(size_t)i * qs + o];
-      return r;
-    };
-    auto combine = [&](const Raw &r) {
-      C v = r.w;
-#pragma unroll
-      for (int i = 0; i < NV; ++i) v = csub(v, cmul(c[i], r.q[i]));
-      return v;
-    };
-    const Raw rprev = load(x, y0 - 1), rcur = load(x, y0), rnext = load(x, y0 + 1);
-    C prev = combine(rprev), cur = combine(rcur), next = combine(rnext);
-    C qcur[NV > 0 ? NV : 1], qnext[NV > 0 ? NV : 1];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      qcur[i] = rcur.q[i];
-      qnext[i] = rnext.q[i];
-    }
-    for (int y = y0; y < y1; ++y) {
-      const Raw r2 = load(x, y + 2);
-      C wv = shfl_c(cur, 1, true), ev = shfl_c(cur, 1, false);
-      if (lane == 0) wv = combine(load(x - 1, y));
-      if (lane == 31) ev = combine(load(x + 1, y));
-      if (x < N) {
-        const C Aq = stencil_vals2<R>(L, x, y, cur, wv, ev, prev, next);
-        const size_t o = off + (size_t)y * P + x;
-        if (OA) Q[(size_t)(J + 1) * qs + o] = cur;
-        if (!LAST) w_out[o] = Aq;
-        const C a = cscale(Aq, s_op);
-        if (OA) {
-          const C vs = cscale(cur, s_op);
-          acc[0] += vs.x * vs.x + vs.y * vs.y;
-#pragma unroll
-          for (int i = 0; i < NV; ++i) {
-            const C qi = cscale(qcur[i], sc[i]);
-            acc[1 + 2 * i] += qi.x * a.x + qi.y * a.y;
-            acc[2 + 2 * i] += qi.x * a.y - qi.y * a.x;
-          }
-          acc[NI - 2] += vs.x * a.x + vs.y * a.y;
-          acc[NI - 1] += vs.x * a.y - vs.y * a.x;
-          if (LAST) acc[NQ - 1] += a.x * a.x + a.y * a.y;
-        } else {
-          const C q0s = cscale(cur, s_op);
-          acc[0] += q0s.x * a.x + q0s.y * a.y;
-          acc[1] += q0s.x * a.y - q0s.y * a.x;
-        }
-      }
-      prev = cur;
-      cur = next;
-      next = combine(r2);
-#pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        qcur[i] = qnext[i];
-        qnext[i] = r2.q[i];
-      }
-    }
-  }
-  write_partials<NQ>(acc, act, parts, b);
-  if constexpr (!OA) {
-    last_block_reduce<NQ>(counter, parts, gridDim.x, gridDim.y, st,
-                          [&](int bb, const double *v) {
-                            double *g = gsc + bb * kGmresScalars;
-                            const float s0 = kscale_of<R>(g, 0);
-                            put_c(g, 0, 0, fin_coef<R>(g, 0, v[0], s0, s0),
-                                  fin_coef<R>(g, 0, v[1], s0, s0));
-                          });
-  } else {
-    last_block_reduce<NQ>(counter, parts, gridDim.x, gridDim.y, st,
-                          [&](int bb, const double *v) {
-                            fin_fused<R, J, LAST>(gsc + bb * kGmresScalars, v);
-                          });
-  }
-}
-
-// The start kernel's column-marching version (2-D): q_0 = f - A u, |q_0|^2,
-// the march over u as in k_gm_col2d.  The grid has nblk blocks per
-// right-hand side like the point-wise kernel (level 0's per-block sums are
-// the stop test's); blocks past the last run of rows add nothing.
-template <typename R>
-__global__ void __launch_bounds__(256)
-k_gm_start_col2d(LevelK<R> L, const typename Cx<R>::T *__restrict__ u, int zero_mode,
-                 const typename Cx<R>::T *__restrict__ f, typename Cx<R>::T *__restrict__ q0,
-                 const SolveState *st, double *parts, unsigned int *counter, double *gsc,
-                 int nchunk, int rows) {
-  using C = typename Cx<R>::T;
-  const int b = blockIdx.y;
-  const bool act = __syncthreads_and(!(st && !st[b].active)) != 0;
-  const bool zero =
-      __syncthreads_or(zero_mode == ZERO_ALL || (zero_mode == ZERO_FLAG && st && st[b].zero)) != 0;
-  if (act && blockIdx.x == 0 && threadIdx.x == 0)
-    put_zero(gsc + b * kGmresScalars, zero);   // for the update kernel
-  R acc[1] = {R(0)};
-  const int N = L.N, P = L.P, lane = threadIdx.x & 31;
-  const int runs = (N + rows - 1) / rows;
-  if (act && (int)blockIdx.x < nchunk * runs) {
-    const size_t off = (size_t)b * L.S;
-    const C *ub = u + off;
-    const int chunk = blockIdx.x % nchunk, run = blockIdx.x / nchunk;
-    const int x = chunk * blockDim.x + threadIdx.x;
-    const int y0 = run * rows, y1 = min(N, y0 + rows);
-    auto load = [&](int xx, int yy) {
-      return (zero || xx < 0 || xx >= N || yy < 0 || yy >= N) ? czero<C>() : ub[(size_t)yy * P + xx];
-    };
-    C prev = load(x, y0 - 1), cur = load(x, y0), next = load(x, y0 + 1);
-    for (int y = y0; y < y1; ++y) {
-      const C n2 = load(x, y + 2);
-      C wv = shfl_c(cur, 1, true), ev = shfl_c(cur, 1, false);
-      if (lane == 0) wv = load(x - 1, y);
-      if (lane == 31) ev = load(x + 1, y);
-      if (x < N) {
-        const size_t o = off + (size_t)y * P + x;
-        C r = f[o];
-        if (!zero) r = csub(r, stencil_vals2<R>(L, x, y, cur, wv, ev, prev, next));
-        q0[o] = r;
-        acc[0] += r.x * r.x + r.y * r.y;
-      }
-      prev = cur;
-      cur = next;
-      next = n2;
-    }
-  }
-  write_partials<1>(acc, act, parts, b);
-  last_block_reduce<1>(counter, parts, gridDim.x, gridDim.y, st,
-                       [&](int bb, const double *v) { fin_norm<R>(gsc + bb * kGmresScalars, 0, v[0], 1.f); });
-}
-
 // Least squares min ||beta e1 - H y|| for the Krylov dimension k (m columns
 // at most), by complex Givens rotations; z_j = y_j / |q_j|.
 __device__ void gm_lsq(double *g, int m, double tiny) {
@@ -949,49 +723,15 @@ k_gm_correct(LevelK<R> L, const typename Cx<R>::T *u_in, const typename Cx<R>::T
 
 // ---------------------------------------------------------------------------
 // The GMRES-smoothed cycle of the small levels in one block per right-hand
-// side.  Shared memory: per level its iterate U, right-hand side F,
-// coefficient tables and k^2 (the level's LevelK is re-pointed at these
-// copies, so the stencil arithmetic is that of the per-level kernels); the
-// Krylov vectors q_0..q_2 are shared by the levels, since a coarser level
-// runs only between a finer level's smoothing steps.  A q_J is not stored:
-// it is recomputed for the inner products and again for the
-// orthogonalisation.  Reductions are FP64 block sums in a fixed order.
+// side, one reduction per step (hh_cheb.cuh).  Shared memory: per level its
+// iterate U, right-hand side F, coefficient tables and k^2 (the level's LevelK
+// is re-pointed at these copies, so the stencil arithmetic is that of the
+// per-level kernels); the vectors q_0..q_2 are shared by the levels, since a
+// coarser level runs only between a finer level's smoothing steps.  Rows have
+// the pitch N + 1, a power of two, so that a thread gets its points'
+// coordinates by shifts.
 // ---------------------------------------------------------------------------
 constexpr int TB = 512;
-
-// Sum the first nq of NQ values per thread over the block, then thread 0 uses
-// the sums (fin) before the block barrier that publishes its results: each
-// warp adds its lanes' values in their own precision into ws (NQ x 32 slots,
-// the first TB / 32 of each row written); warp 0 adds the warp sums (lanes 4q..4q+3 take quantity q, four warp
-// sums each, then two butterfly steps; a fixed order) and its lane 0 runs fin
-// before the block barrier that publishes fin's results.
-template <int NQ, typename A, typename Fin>
-__device__ __forceinline__ void tail_reduce_fin(A (&acc)[NQ], double *ws, double *red, int nq,
-                                                Fin fin) {
-  static_assert(TB / 32 == 16 && NQ <= 8, "16 warps, at most 8 quantities");
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    if (q >= nq) break;
-    A v = acc[q];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) ws[q * 32 + w] = (double)v;
-  }
-  __syncthreads();
-  if (w == 0) {
-    const int q = lane >> 2, part = lane & 3;
-    double v = 0.0;
-    if (q < nq)
-      v = (ws[q * 32 + 4 * part] + ws[q * 32 + 4 * part + 1]) +
-          (ws[q * 32 + 4 * part + 2] + ws[q * 32 + 4 * part + 3]);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    if (part == 0 && q < nq) red[q] = v;
-    __syncwarp();
-    if (lane == 0) fin();
-  }
-  __syncthreads();
-}
 
 template <typename R, int DIM>
 __device__ __forceinline__ LevelK<R> tail_level(const GmTailArgs<R> &A, typename Cx<R>::T *cm,
@@ -1000,216 +740,253 @@ __device__ __forceinline__ LevelK<R> tail_level(const GmTailArgs<R> &A, typename
   const int N = K.N;
   K.coef = cm + A.lv[i].offT;
   K.k2 = km + A.lv[i].offK;
-  K.KP = N;
-  K.P = N;
-  K.S = (long long)npts<DIM>(N);
+  K.KP = N + 1;
+  K.P = N + 1;
+  K.S = (long long)(N + 1) * (DIM == 2 ? N : N * N);
   return K;
 }
 
-// One GMRES(m) step on level K (iterate U, right-hand side F; zero: U is
-// taken as zero).  g: FP64 scalars in the layout of gm_lsq; ws, red: scratch.
-// Every loop over Krylov indices is unrolled to its bound (m <= 3), so the
-// vectors and coefficients stay in registers.
-template <typename R, int DIM>
-__device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T *U,
-                             const typename Cx<R>::T *F, typename Cx<R>::T *Q0,
-                             typename Cx<R>::T *Q1, typename Cx<R>::T *Q2, int m, bool zero,
-                             double *g, double *ws, double *red) {
+// Calls fn(p, x, y, z) for the points of a level that this thread owns (p: the
+// pitched position); the same points in every phase.
+template <int DIM, typename F> __device__ __forceinline__ void tail_points(int N, F fn) {
+  const int lg = 31 - __clz(N + 1);
+  const int total = DIM == 2 ? N << lg : (N * N) << lg;
+  for (int p = threadIdx.x; p < total; p += TB) {
+    const int x = p & N, r = p >> lg;
+    if (x == N) continue;
+    if (DIM == 2) {
+      fn(p, x, r, 0);
+    } else {
+      const int z = r / N;
+      fn(p, x, r - z * N, z);
+    }
+  }
+}
+
+// One GMRES(M) step on level K (iterate U, right-hand side F; zero: U is taken
+// as zero).  res: Q0 holds f - A u of the new iterate afterwards.
+template <typename R, int DIM, int M>
+__device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s,
+                             typename Cx<R>::T *U, const typename Cx<R>::T *F,
+                             typename Cx<R>::T *Q0, typename Cx<R>::T *Q1, typename Cx<R>::T *Q2,
+                             bool zero, bool res,
+                             typename GramSum<R>::T *sums, StepCoef<R> *sc) {
   using C = typename Cx<R>::T;
-  const int N = K.N;
-  const int npt = (int)npts<DIM>(N);
-  const double tiny = sizeof(R) == 4 ? 1e-12 : 1e-26;
-  auto Q = [&](int i) { return i == 0 ? Q0 : (i == 1 ? Q1 : Q2); };
-  // q_0 = F - A U, |q_0|^2 (per-thread sums in the vectors' precision)
+  constexpr bool PAIR = sizeof(R) == 4;
+  constexpr int NQP = Gram<M>::NQP;
+  const int N = K.N, P = K.P;
+  const C t = cscale(sigma, s);
+  auto X = [&](const C *q, int x, int y, int z, C &qc) {
+    auto get = [&](int xx, int yy, int zz) { return q[at<DIM>(xx, yy, zz, N, P)]; };
+    C Aq, D;
+    stencil<R, DIM>(K, x, y, z, get, Aq, D, qc);
+    return cscale(csub(Aq, cmul(sigma, qc)), s);
+  };
   {
-    R acc[1] = {R(0)};
-    auto get = [&](int xx, int yy, int zz) { return U[at<DIM>(xx, yy, zz, N, N)]; };
-    for (int p = threadIdx.x; p < npt; p += TB) {
+    auto get = [&](int xx, int yy, int zz) { return U[at<DIM>(xx, yy, zz, N, P)]; };
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) {
       C r = F[p];
       if (!zero) {
-        int x, y, z;
-        coords<DIM>(p, N, x, y, z);
         C Au, D, uc;
         stencil<R, DIM>(K, x, y, z, get, Au, D, uc);
         r = csub(r, Au);
       }
       Q0[p] = r;
-      acc[0] += r.x * r.x + r.y * r.y;
-    }
-    // (every thread reads the scale of q_0 next)
-    tail_reduce_fin<1>(acc, ws, red, 1, [&] { fin_norm<R>(g, 0, red[0], 1.f); });
+    });
   }
+  __syncthreads();
+  if (M >= 2) {
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) {
+      C qc;
+      Q1[p] = X(Q0, x, y, z, qc);
+    });
+    __syncthreads();
+  }
+  if (M >= 3) {
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) {
+      C qc;
+      const C v = X(Q1, x, y, z, qc);
+      Q2[p] = csub(cadd(v, v), Q0[p]);
+    });
+    __syncthreads();
+  }
+  GramAcc<R, PAIR> acc[NQP];
 #pragma unroll
-  for (int J = 0; J < 3; ++J) {
-    if (J >= m) break;
-    const C *qj = Q(J);
-    auto get = [&](int xx, int yy, int zz) { return qj[at<DIM>(xx, yy, zz, N, N)]; };
-    R sc[3];   // scales of q_0..q_J (written before the last barrier)
+  for (int i = 0; i < NQP; ++i) acc[i].zero();
+  tail_points<DIM>(N, [&](int p, int x, int y, int z) {
+    C qc, v[M + 1];
+    const C xl = X(M == 1 ? Q0 : (M == 2 ? Q1 : Q2), x, y, z, qc);
+    v[0] = Q0[p];
+    if (M >= 2) v[1] = cfma(t, v[0], Q1[p]);
+    if (M == 3) v[M - 1] = cfma(t, Q1[p], cscale(cadd(qc, v[0]), R(0.5)));
+    v[M] = cfma(t, qc, xl);
+    gram_point<R, M, PAIR>(acc, v);
+  });
+  constexpr int SH = NQP == 16 ? 1 : 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  {
+    const GramAcc<R, PAIR> v = gram_warp_sum<GramAcc<R, PAIR>, NQP>(acc);
+    if ((lane & ((1 << SH) - 1)) == 0) sums[warp * NQP + (lane >> SH)] = gram_store(v);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    // the warps that own points (the others' sums are zero)
+    const int nw = min(TB / 32, ((int)K.S + 31) / 32);
+    GramAcc<R, PAIR> v;
+    v.zero();
+    for (int i = lane / NQP; i < nw; i += 32 / NQP) gram_add(v, sums[i * NQP + lane % NQP]);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) sc[i] = i <= J ? kscale_of<R>(g, i) : R(0);
-    // <q_i, A q_J> for i <= J; in the last column also |A q_J|^2, from which
-    // |q_m|^2 and the least-squares solve (q_m itself is not formed)
-    const bool last = J + 1 == m;
-    {
-      R acc[7];
+    for (int o = NQP; o < 32; o <<= 1) v.add(v.shfl_xor(o));
+    __syncwarp();
+    if (lane < NQP) sums[lane] = gram_store(v);
+    __syncwarp();
+    gram_solve<R, M>(sums, s, gram_tol<R>(PAIR), sc);
+  }
+  __syncthreads();
+  if constexpr (sizeof(R) == 8) {
+    // small pivot: one step of refinement (see k_gm2d_coef, hh_gmres2d_64.cu)
+    if (sc->pivot < kPivotOk) {
+      using A = GramAcc<double, false>;
+      A cor[8];
 #pragma unroll
-      for (int i = 0; i < 7; ++i) acc[i] = R(0);
-      for (int p = threadIdx.x; p < npt; p += TB) {
-        int x, y, z;
-        coords<DIM>(p, N, x, y, z);
-        C Aq, D, qc;
-        stencil<R, DIM>(K, x, y, z, get, Aq, D, qc);
-        const C a = cscale(Aq, sc[J]);
+      for (int i = 0; i < 8; ++i) cor[i].zero();
+      double2 yc[M];
 #pragma unroll
-        for (int i = 0; i <= J; ++i) {
-          const C qi = cscale(Q(i)[p], sc[i]);
-          acc[2 * i] += qi.x * a.x + qi.y * a.y;
-          acc[2 * i + 1] += qi.x * a.y - qi.y * a.x;
-        }
-        acc[2 * (J + 1)] += a.x * a.x + a.y * a.y;   // used in the last column only
-      }
-      tail_reduce_fin<7>(acc, ws, red, 2 * (J + 1) + (last ? 1 : 0), [&] {
-        for (int i = 0; i <= J; ++i)
-          put_c(g, i, J, fin_coef<R>(g, i, red[2 * i], sc[i], sc[J]),
-                fin_coef<R>(g, i, red[2 * i + 1], sc[i], sc[J]));
-        if (last) {
-          fin_norm_next<R>(g, J, red[2 * (J + 1)], sc[J]);
-          gm_lsq_r<R>(g, m, tiny);
+      for (int j = 0; j < M; ++j) yc[j] = cscale(sc->z[j], 1.0 / s);
+      tail_points<DIM>(N, [&](int p, int x, int y, int z) {
+        C qc, a[M];
+        const C xl = X(M == 1 ? Q0 : (M == 2 ? Q1 : Q2), x, y, z, qc);
+        if (M >= 2) a[0] = cfma(t, Q0[p], Q1[p]);
+        if (M == 3) a[1 % M] = cfma(t, Q1[p], cscale(cadd(qc, Q0[p]), 0.5));
+        a[M - 1] = cfma(t, qc, xl);
+        C r = Q0[p];
+#pragma unroll
+        for (int j = 0; j < M; ++j) r = csub(r, cmul(yc[j], a[j]));
+#pragma unroll
+        for (int j = 0; j < M; ++j) {
+          cor[2 * j].mac(a[j].x, r.x);
+          cor[2 * j].mac(a[j].y, r.y);
+          cor[2 * j + 1].mac(a[j].x, r.y);
+          cor[2 * j + 1].mac(-a[j].y, r.x);
         }
       });
-    }
-    if (last) break;
-    // q_{J+1} = A q_J - sum_i c_iJ q_i (J + 1 < m), |q_{J+1}|^2
-    {
-      C c[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        c[i] = i <= J ? get_c<R>(g, i, J) : czero<C>();
-      R acc[1] = {R(0)};
-      C *qn = Q(J + 1);
-      for (int p = threadIdx.x; p < npt; p += TB) {
-        int x, y, z;
-        coords<DIM>(p, N, x, y, z);
-        C v, D, qc;
-        stencil<R, DIM>(K, x, y, z, get, v, D, qc);
-#pragma unroll
-        for (int i = 0; i <= J; ++i) v = csub(v, cmul(c[i], Q(i)[p]));
-        qn[p] = v;
-        const C vs = cscale(v, sc[J]);
-        acc[0] += vs.x * vs.x + vs.y * vs.y;
+      const A v = gram_warp_sum<A, 8>(cor);
+      double *corr = sums + 16;   // (the warps' sums are used up)
+      if ((lane & 3) == 0) corr[warp * 8 + (lane >> 2)] = v.h;
+      __syncthreads();
+      if (warp == 0) {
+        double q = 0.0;
+        if (lane < 8)
+          for (int w = 0; w < TB / 32; ++w) q += corr[w * 8 + lane];
+        if (lane < 2 * M) sums[Gram<M>::pair(0, lane / 2 + 1) + (lane & 1)] = (lane & 1) ? -q : q;
+        __syncwarp();
+        const C z0 = lane < 3 ? sc->z[lane] : czero<C>();
+        __syncwarp();
+        gram_solve<R, M>(sums, s, gram_tol<R>(PAIR), sc);
+        __syncwarp();
+        if (lane < 3) sc->z[lane] = cadd(z0, sc->z[lane]);
       }
-      tail_reduce_fin<1>(acc, ws, red, 1, [&] { fin_norm<R>(g, J + 1, red[0], sc[J]); });
+      __syncthreads();
     }
   }
-  // U = U + sum_j z_j q_j
-  {
-    const int k = min(m, get_k(g));
-    C z[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) z[j] = get_z<R>(g, j);
-    for (int p = threadIdx.x; p < npt; p += TB) {
-      C v = zero ? czero<C>() : U[p];
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        if (j < k) v = cfma(z[j], Q(j)[p], v);
-      U[p] = v;
-    }
+  tail_points<DIM>(N, [&](int p, int, int, int) {
+    C v = zero ? czero<C>() : U[p];
+    v = cfma(sc->z[0], Q0[p], v);
+    if (M >= 2) v = cfma(sc->z[1], Q1[p], v);
+    if (M >= 3) v = cfma(sc->z[2], Q2[p], v);
+    U[p] = v;
+  });
+  __syncthreads();
+  if (res) {
+    auto get = [&](int xx, int yy, int zz) { return U[at<DIM>(xx, yy, zz, N, P)]; };
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) {
+      C Au, D, uc;
+      stencil<R, DIM>(K, x, y, z, get, Au, D, uc);
+      Q0[p] = csub(F[p], Au);
+    });
     __syncthreads();
   }
 }
 
-template <typename R, int DIM>
+template <typename R, int DIM, int M>
 __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailArgs<R> A,
                                                 const SolveState *st) {
   using C = typename Cx<R>::T;
   const int b = blockIdx.x;
-  if (!__syncthreads_and(!(st && !st[b].active))) return;   // one decision per block
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *cm = reinterpret_cast<C *>(smem_raw);
   R *km = reinterpret_cast<R *>(smem_raw + A.kbase);
   double2 *slu = reinterpret_cast<double2 *>(smem_raw + A.lubase);
   const int mm = A.mm;
   int *spiv = reinterpret_cast<int *>(slu + mm * mm);
-  __shared__ double g[kGmresScalars];
-  __shared__ double ws[7 * 32];
-  __shared__ double red[7];
+  // (complex128: room for the refinement's sums behind the Gram matrix)
+  __shared__ typename GramSum<R>::T sums[sizeof(R) == 8 ? 16 + (TB / 32) * 16 : (TB / 32) * Gram<M>::NQP];
+  __shared__ StepCoef<R> sc;
   C *const Q0 = cm + A.offQ[0], *const Q1 = cm + A.offQ[1], *const Q2 = cm + A.offQ[2];
-  // stage the top right-hand side, every level's tables and k^2, the LU
-  {
-    const int N = A.lv[0].K.N;
-    const C *fb = A.f + (size_t)b * A.lay.S;
-    C *F = cm + A.lv[0].offF;
-    for (int p = threadIdx.x; p < (int)npts<DIM>(N); p += TB) {
-      int x, y, z;
-      coords<DIM>(p, N, x, y, z);
-      F[p] = fb[at<DIM>(x, y, z, N, A.lay.P)];
-    }
-  }
+  // every level's tables and k^2 and the LU, which no kernel writes: staged
+  // before the dependency wait
   for (int i = 0; i < A.nl; ++i) {
     const LevelK<R> &G = A.lv[i].K;
     const int N = G.N;
     C *tab = cm + A.lv[i].offT;
     for (int j = threadIdx.x; j < 3 * DIM * N; j += TB) tab[j] = G.coef[j];
     R *kk = km + A.lv[i].offK;
-    for (int p = threadIdx.x; p < (int)npts<DIM>(N); p += TB) {
-      int x, y, z;
-      coords<DIM>(p, N, x, y, z);
-      kk[p] = G.k2[at<DIM>(x, y, z, N, G.KP)];
-    }
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) { kk[p] = G.k2[at<DIM>(x, y, z, N, G.KP)]; });
   }
   for (int j = threadIdx.x; j < mm * mm; j += TB) slu[j] = A.lu[j];
   for (int j = threadIdx.x; j < mm; j += TB) spiv[j] = A.piv[j];
+  griddep_wait();
+  griddep_launch_dependents();
+  if (!__syncthreads_and(!(st && !st[b].active))) return;   // one decision per block
+  {
+    const int N = A.lv[0].K.N;
+    const C *fb = A.f + (size_t)b * A.lay.S;
+    C *F = cm + A.lv[0].offF;
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) { F[p] = fb[at<DIM>(x, y, z, N, A.lay.P)]; });
+  }
   __syncthreads();
-  // way down: smoothing from zero, residual, full weighting
+  // way down: smoothing from zero, full weighting of the last step's residual
   for (int i = 0; i + 1 < A.nl; ++i) {
     const LevelK<R> K = tail_level<R, DIM>(A, cm, km, i);
-    const int N = K.N, Nc = A.lv[i + 1].K.N;
+    const int N = K.N, P = K.P, Nc = A.lv[i + 1].K.N;
     C *U = cm + A.lv[i].offU;
     const C *F = cm + A.lv[i].offF;
     for (int s = 0; s < A.nu1; ++s)
-      tail_gm_step<R, DIM>(K, U, F, Q0, Q1, Q2, A.m, s == 0, g, ws, red);
-    {
-      auto get = [&](int xx, int yy, int zz) { return U[at<DIM>(xx, yy, zz, N, N)]; };
-      for (int p = threadIdx.x; p < (int)npts<DIM>(N); p += TB) {
-        int x, y, z;
-        coords<DIM>(p, N, x, y, z);
-        C Au, D, uc;
-        stencil<R, DIM>(K, x, y, z, get, Au, D, uc);
-        Q0[p] = csub(F[p], Au);
-      }
-    }
-    __syncthreads();
+      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, U, F, Q0, Q1, Q2, s == 0,
+                              s == A.nu1 - 1, sums, &sc);
     {
       const C *r = Q0;
       C *Fc = cm + A.lv[i + 1].offF;
       const int zlo = DIM == 3 ? -1 : 0, zhi = DIM == 3 ? 1 : 0;
       const R scale = DIM == 3 ? R(1.0 / 64.0) : R(1.0 / 16.0);
       const C cs = A.lv[i].c;
-      for (int pc = threadIdx.x; pc < (int)npts<DIM>(Nc); pc += TB) {
-        int cx, cy, cz;
-        coords<DIM>(pc, Nc, cx, cy, cz);
-        C acc = czero<C>();
+      tail_points<DIM>(Nc, [&](int, int cx, int cy, int cz) {
+        C a = czero<C>();
         for (int dz = zlo; dz <= zhi; ++dz)
+#pragma unroll
           for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
             for (int dx = -1; dx <= 1; ++dx) {
               const int x = 2 * cx + 1 + dx, y = 2 * cy + 1 + dy;
               const int z = DIM == 3 ? 2 * cz + 1 + dz : 0;
               const R w = R((2 - abs(dx)) * (2 - abs(dy)) * (DIM == 3 ? 2 - abs(dz) : 1));
-              acc = cadd(acc, cscale(r[at<DIM>(x, y, z, N, N)], w));
+              a = cadd(a, cscale(r[at<DIM>(x, y, z, N, P)], w));
             }
-        Fc[pc] = cmul(cs, cscale(acc, scale));
-      }
+        Fc[at<DIM>(cx, cy, cz, Nc, Nc + 1)] = cmul(cs, cscale(a, scale));
+      });
     }
     __syncthreads();
   }
   // coarsest level: LU substitution (FP64) by one warp, lane i owning row i
   if (threadIdx.x < 32) {
-    const int i = threadIdx.x;
+    const int i = threadIdx.x, N = A.lv[A.nl - 1].K.N;
     const C *fl = cm + A.lv[A.nl - 1].offF;
     C *ul = cm + A.lv[A.nl - 1].offU;
     double2 y = make_double2(0.0, 0.0);
+    int x, yy, z;
     if (i < mm) {
-      const C q = fl[spiv[i]];
+      coords<DIM>((size_t)spiv[i], N, x, yy, z);
+      const C q = fl[at<DIM>(x, yy, z, N, N + 1)];
       y = make_double2((double)q.x, (double)q.y);
     }
     for (int k = 0; k < mm; ++k) {
@@ -1221,7 +998,10 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
       const double2 yk = make_double2(__shfl_sync(0xffffffffu, y.x, k), __shfl_sync(0xffffffffu, y.y, k));
       if (i < k) y = csub(y, cmul(slu[i * mm + k], yk));
     }
-    if (i < mm) ul[i] = cmk((R)y.x, (R)y.y);
+    if (i < mm) {
+      coords<DIM>((size_t)i, N, x, yy, z);
+      ul[at<DIM>(x, yy, z, N, N + 1)] = cmk((R)y.x, (R)y.y);
+    }
   }
   __syncthreads();
   // way up: interpolated correction, smoothing
@@ -1231,38 +1011,37 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
     C *U = cm + A.lv[i].offU;
     const C *F = cm + A.lv[i].offF;
     const C *E = cm + A.lv[i + 1].offU;
-    const Lay lc{Nc, Nc, (long long)npts<DIM>(Nc)};
-    for (int p = threadIdx.x; p < (int)npts<DIM>(N); p += TB) {
-      int x, y, z;
-      coords<DIM>(p, N, x, y, z);
+    const Lay lc{Nc, Nc + 1, 0};
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) {
       U[p] = cadd(U[p], prolong_at<R, DIM>(E, lc, x, y, z));
-    }
+    });
     __syncthreads();
     for (int s = 0; s < A.nu2; ++s)
-      tail_gm_step<R, DIM>(K, U, F, Q0, Q1, Q2, A.m, false, g, ws, red);
+      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, U, F, Q0, Q1, Q2, false, false,
+                              sums, &sc);
   }
   {
     const int N = A.lv[0].K.N;
     C *ub = A.u + (size_t)b * A.lay.S;
     const C *U = cm + A.lv[0].offU;
-    for (int p = threadIdx.x; p < (int)npts<DIM>(N); p += TB) {
-      int x, y, z;
-      coords<DIM>(p, N, x, y, z);
-      ub[at<DIM>(x, y, z, N, A.lay.P)] = U[p];
-    }
+    tail_points<DIM>(N, [&](int p, int x, int y, int z) { ub[at<DIM>(x, y, z, N, A.lay.P)] = U[p]; });
   }
 }
 
 }  // namespace
 
+// Shared memory of the tail (layout of setup_gmres_tail): q_0..q_2 of the first
+// level, per level iterate, right-hand side, tables and k^2 (rows
+// of pitch N + 1), the coarsest LU and its pivots.
+static size_t tail_pts(int dim, int N) { return (size_t)(N + 1) * (dim == 2 ? N : N * N); }
 template <typename R, int DIM> size_t gmres_tail_smem(const int *N, int nl, int m) {
   (void)m;
   using C = typename Cx<R>::T;
-  size_t c = 3 * npts<DIM>(N[0]);          // q_0..q_2
+  size_t c = 3 * tail_pts(DIM, N[0]);
   size_t r = 0;
   for (int i = 0; i < nl; ++i) {
-    c += 2 * npts<DIM>(N[i]) + 3 * DIM * (size_t)N[i];
-    r += npts<DIM>(N[i]);
+    c += 2 * tail_pts(DIM, N[i]) + 3 * DIM * (size_t)N[i];
+    r += tail_pts(DIM, N[i]);
   }
   const size_t kb = (c * sizeof(C) + 15) / 16 * 16;
   const size_t lb = (kb + r * sizeof(R) + 15) / 16 * 16;
@@ -1271,29 +1050,27 @@ template <typename R, int DIM> size_t gmres_tail_smem(const int *N, int nl, int 
 }
 
 template <typename R, int DIM> cudaError_t init_gmres_tail() {
-  return cudaFuncSetAttribute(k_gm_tail<R, DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kGmTailSmemMax);
+  cudaError_t e;
+  auto set = [](auto k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmTailSmemMax);
+  };
+  if ((e = set(k_gm_tail<R, DIM, 1>)) != cudaSuccess) return e;
+  if ((e = set(k_gm_tail<R, DIM, 2>)) != cudaSuccess) return e;
+  return set(k_gm_tail<R, DIM, 3>);
 }
 
 template <typename R, int DIM>
 void launch_gmres_tail(const GmTailArgs<R> &a, int batch, const SolveState *st, cudaStream_t s) {
-  k_gm_tail<R, DIM><<<batch, TB, a.smem_bytes, s>>>(a, st);
+  auto go = [&](auto k) { launch_pdl(k, dim3(batch), dim3(TB), a.smem_bytes, s, a, st); };
+  if (a.m == 1) go(k_gm_tail<R, DIM, 1>);
+  else if (a.m == 2) go(k_gm_tail<R, DIM, 2>);
+  else go(k_gm_tail<R, DIM, 3>);
 }
 
 template <typename R, int DIM>
 void launch_gmres_start(const LevelK<R> &L, const typename Cx<R>::T *u, int zero_mode,
                         const typename Cx<R>::T *f, const GmresWork<R> &g, int batch,
-                        const SolveState *st, double *parts, int nblk, cudaStream_t s, int col) {
-  if constexpr (DIM == 2) {
-    if (col) {
-      const int nchunk = (L.N + 255) / 256;
-      const int per = std::max(1, nblk / nchunk);
-      const int rows = (L.N + per - 1) / per;
-      launch_plain(k_gm_start_col2d<R>, dim3(nblk, batch), dim3(256), 0, s, L, u, zero_mode, f,
-                   g.Q, st, parts, g.counter, g.gsc, nchunk, rows);
-      return;
-    }
-  }
+                        const SolveState *st, double *parts, int nblk, cudaStream_t s) {
   launch_plain(k_gm_start<R, DIM>, dim3(nblk, batch), dim3(256), 0, s, L, u, zero_mode, f, g.Q, st,
              parts, g.counter, g.gsc);
 }
@@ -1305,28 +1082,6 @@ void launch_gmres_rest(const LevelK<R> &L, const typename Cx<R>::T *u_in, int ze
   const dim3 grid(nblk, batch);
   const dim3 blk(256);
   using C = typename Cx<R>::T;
-  if constexpr (DIM == 2) {
-    // large levels: the column-marching Arnoldi 0 and fused steps (fuse bit 1)
-    if ((fuse & 1) && (fuse & 2) && m >= 2) {
-      const int nchunk = (L.N + 255) / 256;
-      const int per = std::max(1, nblk / nchunk);   // row runs per chunk (blocks <= nblk)
-      const int rows = (L.N + per - 1) / per;
-      const dim3 gcol(nchunk * ((L.N + rows - 1) / rows), batch);
-      launch_plain(k_gm_col2d<R, false, 0, false>, gcol, blk, 0, s, L, g.Q, g.qs,
-                   (const C *)nullptr, g.w, st, g.parts, g.counter, g.gsc, nchunk, rows);
-      if (m == 2) {
-        launch_plain(k_gm_col2d<R, true, 0, true>, gcol, blk, 0, s, L, g.Q, g.qs, (const C *)g.w,
-                     g.w2, st, g.parts, g.counter, g.gsc, nchunk, rows);
-      } else {
-        launch_plain(k_gm_col2d<R, true, 0, false>, gcol, blk, 0, s, L, g.Q, g.qs,
-                     (const C *)g.w, g.w2, st, g.parts, g.counter, g.gsc, nchunk, rows);
-        launch_plain(k_gm_col2d<R, true, 1, true>, gcol, blk, 0, s, L, g.Q, g.qs,
-                     (const C *)g.w2, g.w, st, g.parts, g.counter, g.gsc, nchunk, rows);
-      }
-      launch_plain(k_gm_update<R, DIM>, grid, blk, 0, s, L, u_in, g.Q, g.qs, u_out, st, g.gsc, m);
-      return;
-    }
-  }
   if ((fuse & 1) && m >= 2) {
     // A q_0 -> w; (q_1, A q_1) -> w2; for m = 3 (q_2, A q_2), whose product
     // only enters |q_3|^2 and the least-squares solve
@@ -1378,8 +1133,7 @@ void launch_gmres_correct(const LevelK<R> &L, const typename Cx<R>::T *u_in,
 #define HH_GMRES_INST(R, DIM)                                                                  \
   template void launch_gmres_start<R, DIM>(const LevelK<R> &, const Cx<R>::T *, int,           \
                                            const Cx<R>::T *, const GmresWork<R> &, int,        \
-                                           const SolveState *, double *, int, cudaStream_t,    \
-                                           int);                                               \
+                                           const SolveState *, double *, int, cudaStream_t);   \
   template void launch_gmres_rest<R, DIM>(const LevelK<R> &, const Cx<R>::T *, int,            \
                                           Cx<R>::T *, const GmresWork<R> &, int, int,          \
                                           const SolveState *, int, cudaStream_t, int);         \
@@ -1395,9 +1149,7 @@ HH_GMTAIL_INST(float, 2)
 HH_GMTAIL_INST(float, 3)
 HH_GMTAIL_INST(double, 2)
 HH_GMTAIL_INST(double, 3)
-HH_GMRES_INST(float, 2)
 HH_GMRES_INST(float, 3)
-HH_GMRES_INST(double, 2)
 HH_GMRES_INST(double, 3)
 
 }  // namespace hh

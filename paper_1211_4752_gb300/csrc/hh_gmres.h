@@ -1,6 +1,7 @@
 // GMRES(m) smoothing kernels (hh_gmres.cu): workspace and launchers.
 #pragma once
 #include "hh_internal.h"
+#include "hh_cheb.cuh"
 
 namespace hh {
 
@@ -24,21 +25,18 @@ template <typename R> struct GmresWork {
 };
 
 // q_0 = f - A u and |q_0|^2; parts (layout [b][block], nblk blocks) may be the
-// stop test's partial sums on level 0.  col (2-D): the column-marching kernel.
+// stop test's partial sums on level 0.
 template <typename R, int DIM>
 void launch_gmres_start(const LevelK<R> &L, const typename Cx<R>::T *u, int zero_mode,
                         const typename Cx<R>::T *f, const GmresWork<R> &g, int batch,
-                        const SolveState *st, double *parts, int nblk, cudaStream_t s,
-                        int col = 0);
+                        const SolveState *st, double *parts, int nblk, cudaStream_t s);
 
 // The m Arnoldi steps, the least-squares solve and u_out = u_in + V y (u_in
 // read as zero where the start kernel took it as zero): 2 m kernels (Arnoldi
 // products, the orthogonalisations of columns 0..m-2, the update; the last
 // Arnoldi kernel forms |q_m| and solves the least-squares problem).  fuse
 // bit 0 (m >= 2): the orthogonalisation of step J and the Arnoldi product of
-// step J+1 in one kernel (m + 1 kernels); bit 1 (2-D): those kernels and
-// Arnoldi step 0 march down columns (hh_gmres.cu, k_gm_col2d; the caller sets
-// it on large levels).
+// step J+1 in one kernel (m + 1 kernels).  3-D levels (2-D: hh_gmres2d.h).
 template <typename R, int DIM>
 void launch_gmres_rest(const LevelK<R> &L, const typename Cx<R>::T *u_in, int zero_mode,
                        typename Cx<R>::T *u_out, const GmresWork<R> &g, int m, int batch,
@@ -60,14 +58,16 @@ constexpr int kGmTailMax = 8;
 template <typename R> struct GmTailLevel {
   LevelK<R> K;                 // the level (tables and k^2 in global memory)
   typename Cx<R>::T c;         // scale of the residual restricted from it
+  typename Cx<R>::T sigma;     // centre and inverse half width of its spectrum
+  R s;                         // (hh_cheb.cuh)
   int offU, offF, offT;        // complex offsets in shared memory: iterate,
                                // right-hand side, coefficient tables (3 dim N)
-  int offK;                    // real offset of k^2 (N^dim)
+  int offK;                    // real offset of k^2
 };
 template <typename R> struct GmTailArgs {
   int nl, m, nu1, nu2;
   GmTailLevel<R> lv[kGmTailMax];
-  int offQ[3];                 // Krylov vectors q_0..q_2 (sized for level t0)
+  int offQ[3];                 // q_0..q_2 (sized for level t0)
   int kbase, lubase, smem_bytes;
   const typename Cx<R>::T *f;  // right-hand side of level t0 (library layout lay)
   typename Cx<R>::T *u;        // its correction
