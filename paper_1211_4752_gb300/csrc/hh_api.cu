@@ -11,6 +11,7 @@
 #include "hh_cycle.h"
 #include "hh_gmres.h"
 #include "hh_gmres2d.h"
+#include "hh_gmres3d.h"
 #include "hh_krylov.h"
 #include "hh_tiled3d.h"
 
@@ -75,9 +76,7 @@ template <typename R> struct Work {
   C *u_post[MAXL] = {};
   C *f[MAXL] = {};
   C *tmp[MAXL] = {};
-  C *gq[MAXL] = {};   // GMRES smoothing: Krylov vectors q_0..q_3 of the level
-  C *gw[MAXL] = {};   // and w = A q_j (two buffers)
-  C *gw2[MAXL] = {};
+  C *gq[MAXL] = {};   // GMRES smoothing: stored vectors of the level's basis
 };
 
 struct LevelHost {
@@ -115,6 +114,7 @@ struct hh_handle {
   std::vector<LevelHost> lv;
   double2 *lu[2] = {nullptr, nullptr};
   int *piv[2] = {nullptr, nullptr};
+  double2 *inv[2] = {nullptr, nullptr};  // inverse of the coarsest operator (GMRES tail)
   Work<double> w64;
   Work<float> w32;
   double2 *u64[2] = {nullptr, nullptr};
@@ -141,10 +141,8 @@ struct hh_handle {
   int ngroups = 0;
   CoarseGroup groups[MAXL];
   int parts_cap = 0;                // capacity of `partials` per RHS
-  int gm_cap = 0;                   // most blocks of a GMRES smoothing kernel
-  int gm_fuse = 1;                  // 3-D: fused orthogonalisation + Arnoldi kernels
   int sms = 0;                      // SMs of the device
-  void *gm2_parts = nullptr;        // 2-D: partial Gram matrices of a step,
+  void *gm2_parts = nullptr;        // GMRES smoothing: partial Gram matrices of a step,
   int *gm2_zero = nullptr;          // whether it started from zero (per right-hand side),
   double *gm2_coef = nullptr;       // complex128: coefficients and their correction's sums
   double *gm2_parts2 = nullptr;
@@ -167,9 +165,6 @@ struct hh_handle {
   PersistArgs pargs[2];             // its arguments per direction (per-call fields filled at launch)
   unsigned int *pbar = nullptr;     // its grid barrier (arrivals, generation)
   int *pskip = nullptr;             // its test hook word (hh_test_barrier_timeout)
-  double *gm_parts = nullptr;       // GMRES smoothing: partial sums,
-  unsigned int *gm_counter = nullptr;  // last-block arrival counter,
-  double *gm_gsc = nullptr;         // per right-hand side scalars
   int gtail0 = 0;                   // GMRES smoothing: first level of the one-block tail (0: none)
   GmTailArgs<float> gta32[2];       // its arguments per direction and precision
   GmTailArgs<double> gta64[2];
@@ -332,32 +327,10 @@ inline bool stop_test(int check) { return check == CHECK_CYCLE || check == CHECK
 // the environment selects the point-wise kernels instead (for comparisons).
 bool pointwise3d(const hh_handle *h) { return h->pw3d != 0; }
 
-template <typename R> GmresWork<R> gmres_work(hh_handle *h, int l) {
-  Work<R> &W = work<R>(h);
-  GmresWork<R> g;
-  g.Q = W.gq[l];
-  g.qs = (size_t)h->lv[l].S * h->max_batch;
-  g.w = W.gw[l];
-  g.w2 = W.gw2[l];
-  g.parts = h->gm_parts;
-  g.counter = h->gm_counter;
-  g.gsc = h->gm_gsc;
-  return g;
-}
-// Blocks of the GMRES smoothing kernels on level l (grid-stride loops of 256
-// threads, at most gm_cap; one partial sum per block and quantity).
-int gmres_blocks(const hh_handle *h, int l) {
-  const size_t g = (h->lv[l].pts + 255) / 256;
-  return (int)std::max<size_t>(1, std::min<size_t>(g, (size_t)h->gm_cap));
-}
-int partial_blocks_of(const hh_handle *h, int l) {
-  return l == 0 ? h->nparts : gmres_blocks(h, l);
-}
-
 int tune_batch(const hh_handle *h);
 void fork_check(hh_handle *h, int check, unsigned long long cond, cudaStream_t s);
 
-// 2-D GMRES steps (hh_gmres2d.h): constants of a level, workspace and split.
+// GMRES steps (hh_gmres2d.h, hh_gmres3d.h): constants of a level, workspace and split.
 template <typename R> struct Gm2dLevel {
   LevelK<R> K;
   typename Cx<R>::T sigma;
@@ -385,15 +358,34 @@ template <typename R> Gm2dPlan gm2d_plan_of(const hh_handle *h, int l, bool rest
   return gm2d_plan<R>(h->lv[l].N, h->opt.gmres_m, tune_batch(h), h->sms, restrict_);
 }
 
-// One GMRES step on level l (2-D): u_out = in + z; with fc the restricted
-// residual of u_out as well.
+Gm3dPlan gm3d_plan_of(const hh_handle *h, int l) {
+  return gm3d_plan(h->lv[l].N, tune_batch(h), h->sms);
+}
+
+// One GMRES step on level l: u_out = in + z; restrict_: the restricted residual of
+// u_out as well.
 template <typename R>
-void enqueue_gm2d_step(hh_handle *h, int l, int dir, const Gm2dIn<R> &in, typename Cx<R>::T *u_out,
+void enqueue_gm_step(hh_handle *h, int l, int dir, const Gm2dIn<R> &in, typename Cx<R>::T *u_out,
                        bool restrict_, int batch, const SolveState *st, int check,
                        unsigned long long cond, cudaStream_t s) {
   const Gm2dLevel<R> g = gm2d_level<R>(h, l, dir);
-  const Gm2dPlan p = gm2d_plan_of<R>(h, l, restrict_);
   const int m = h->opt.gmres_m;
+  if (h->dim == 3) {
+    const Gm3dPlan p = gm3d_plan_of(h, l);
+    launch_gm3d_basis<R>(g.K, g.sigma, g.s, h->kconst, m, in, g.w, p, u_out, batch, st,
+                         stop_test(check) ? h->partials : nullptr, s);
+    if (stop_test(check)) fork_check(h, check, cond, s);
+    launch_gm3d_update<R>(g.K, g.sigma, g.s, m, in, g.w, p, u_out, batch, st, s);
+    if (!restrict_) return;
+    if (pointwise3d(h))
+      launch_resid_restrict<R, 3>(g.K, u_out, work<R>(h).f[l], work<R>(h).f[l + 1], lay_of(h, l + 1),
+                                  cscal<R>(h, l, dir), batch, st, s);
+    else
+      launch_resid_restrict3d<R>(g.K, u_out, work<R>(h).f[l], work<R>(h).f[l + 1], lay_of(h, l + 1),
+                                 cscal<R>(h, l, dir), batch, st, s);
+    return;
+  }
+  const Gm2dPlan p = gm2d_plan_of<R>(h, l, restrict_);
   launch_gm2d_basis<R>(g.K, g.sigma, g.s, h->kconst, m, in, g.w, p, batch, st,
                        stop_test(check) ? h->partials : nullptr, s);
   if (stop_test(check)) fork_check(h, check, cond, s);
@@ -412,14 +404,14 @@ void enqueue_gmres_tail(hh_handle *h, int dir, int batch, const SolveState *st, 
   else go(h->gta64[dir]);
 }
 
-// The 2-D V-cycle with GMRES(m) smoothing: two kernels per step; the last
-// pre-smoothing step restricts its residual, the first post-smoothing step
-// starts from the corrected iterate.  On level 0 the first step's |f - A u|^2
+// The V-cycle with GMRES(m) smoothing (Sec. 3.2): the last pre-smoothing step
+// restricts its residual, the first post-smoothing step starts from the corrected
+// iterate.  On level 0 the first step's |f - A u|^2
 // is the stop test's, which runs on a branch beside the coarser levels and is
 // joined before the one part of the cycle that writes the level-0 iterate (the
 // level-0 post-smoothing; see fork_check).
 template <typename R>
-void enqueue_cycle_gmres2d(hh_handle *h, int dir, int batch, int zero0, int check,
+void enqueue_cycle_gmres(hh_handle *h, int dir, int batch, int zero0, int check,
                            unsigned long long cond, cudaStream_t s) {
   using C = typename Cx<R>::T;
   Work<R> &W = work<R>(h);
@@ -432,7 +424,7 @@ void enqueue_cycle_gmres2d(hh_handle *h, int dir, int batch, int zero0, int chec
     for (int j = 0; j < nu1; ++j) {
       C *out = (nu1 - 1 - j) % 2 == 0 ? W.u_pre[l] : W.tmp[l];
       const Gm2dIn<R> a{in, W.f[l], nullptr, Lay{0, 0, 0}, zm};
-      enqueue_gm2d_step<R>(h, l, dir, a, out, j == nu1 - 1, batch, st,
+      enqueue_gm_step<R>(h, l, dir, a, out, j == nu1 - 1, batch, st,
                            l == 0 && j == 0 ? check : CHECK_NONE, cond, s);
       in = out;
       zm = ZERO_NONE;
@@ -441,73 +433,16 @@ void enqueue_cycle_gmres2d(hh_handle *h, int dir, int batch, int zero0, int chec
   if (h->gtail0 > 0)
     enqueue_gmres_tail<R>(h, dir, batch, st, s);
   else
-    launch_coarse_solve<R, 2>(h->lu[dir], h->piv[dir], lay_of(h, L - 1), W.f[L - 1],
-                              W.u_post[L - 1], batch, st, s);
+    (h->dim == 2 ? launch_coarse_solve<R, 2> : launch_coarse_solve<R, 3>)(
+        h->lu[dir], h->piv[dir], lay_of(h, L - 1), W.f[L - 1], W.u_post[L - 1], batch, st, s);
   for (int l = T - 1; l >= 0; --l) {
     if (l == 0 && stop_test(check)) cudaStreamWaitEvent(s, h->ev_join, 0);
     const C *in = W.u_pre[l];
     for (int j = 0; j < nu2; ++j) {
       C *out = (nu2 - 1 - j) % 2 == 0 ? W.u_post[l] : W.tmp[l];
       const Gm2dIn<R> a{in, W.f[l], j == 0 ? W.u_post[l + 1] : nullptr, lay_of(h, l + 1), ZERO_NONE};
-      enqueue_gm2d_step<R>(h, l, dir, a, out, false, batch, st, CHECK_NONE, cond, s);
+      enqueue_gm_step<R>(h, l, dir, a, out, false, batch, st, CHECK_NONE, cond, s);
       in = out;
-    }
-  }
-}
-
-// The 3-D V-cycle with GMRES(m) smoothing (Sec. 3.2): on each level nu1 GMRES
-// steps, residual + restriction, recursion, correction, nu2 GMRES steps.
-// On level 0 the first step's residual is the stop test's.
-template <typename R>
-void enqueue_cycle_gmres3d(hh_handle *h, int dir, int batch, int zero0, int check,
-                         unsigned long long cond, cudaStream_t s) {
-  constexpr int DIM = 3;
-  Work<R> &W = work<R>(h);
-  const SolveState *st = check != CHECK_NONE ? h->st : nullptr;
-  const int L = h->L, m = h->opt.gmres_m;
-  // levels gtail0 .. coarsest run in one block per right-hand side
-  const int T = h->gtail0 > 0 ? h->gtail0 : L - 1;
-  for (int l = 0; l < T; ++l) {
-    const LevelK<R> K = levelk<R>(h, l, dir);
-    const GmresWork<R> g = gmres_work<R>(h, l);
-    const int nb = partial_blocks_of(h, l);
-    const typename Cx<R>::T *in = l == 0 ? W.u_post[0] : W.u_pre[l];
-    int zm = l == 0 ? zero0 : ZERO_ALL;
-    for (int j = 0; j < h->opt.nu1; ++j) {
-      const bool norm = l == 0 && j == 0 && stop_test(check);
-      launch_gmres_start<R, DIM>(K, in, zm, W.f[l], g, batch, st, norm ? h->partials : g.parts, nb, s);
-      if (norm) {
-        if (check == CHECK_CYCLE)
-          launch_check_cycle(h->st, h->partials, h->params, h->flag, cond, h->copies, h->err, s);
-        else
-          launch_check_inner(h->st, h->partials, h->params, h->flag, cond, h->copies, h->err, s);
-      }
-      launch_gmres_rest<R, DIM>(K, in, zm, W.u_pre[l], g, m, batch, st, nb, s, h->gm_fuse);
-      in = W.u_pre[l];
-      zm = ZERO_NONE;
-    }
-    if (!pointwise3d(h))
-      launch_resid_restrict3d<R>(K, W.u_pre[l], W.f[l], W.f[l + 1], lay_of(h, l + 1),
-                                 cscal<R>(h, l, dir), batch, st, s);
-    else
-      launch_resid_restrict<R, DIM>(K, W.u_pre[l], W.f[l], W.f[l + 1], lay_of(h, l + 1),
-                                    cscal<R>(h, l, dir), batch, st, s);
-  }
-  if (h->gtail0 > 0) {
-    enqueue_gmres_tail<R>(h, dir, batch, st, s);
-  } else {
-    launch_coarse_solve<R, DIM>(h->lu[dir], h->piv[dir], lay_of(h, L - 1), W.f[L - 1],
-                                W.u_post[L - 1], batch, st, s);
-  }
-  for (int l = T - 1; l >= 0; --l) {
-    const LevelK<R> K = levelk<R>(h, l, dir);
-    const GmresWork<R> g = gmres_work<R>(h, l);
-    const int nb = partial_blocks_of(h, l);
-    launch_gmres_correct<R, DIM>(K, W.u_pre[l], W.u_post[l + 1], lay_of(h, l + 1), W.u_post[l],
-                                 batch, st, s);
-    for (int j = 0; j < h->opt.nu2; ++j) {
-      launch_gmres_start<R, DIM>(K, W.u_post[l], ZERO_NONE, W.f[l], g, batch, st, g.parts, nb, s);
-      launch_gmres_rest<R, DIM>(K, W.u_post[l], ZERO_NONE, W.u_post[l], g, m, batch, st, nb, s, h->gm_fuse);
     }
   }
 }
@@ -516,8 +451,7 @@ template <typename R, int DIM>
 void enqueue_cycle(hh_handle *h, int dir, int batch, int zero0, int check,
                    unsigned long long cond, cudaStream_t s) {
   if (h->opt.smoother == HH_SMOOTH_GMRES) {
-    if constexpr (DIM == 2) enqueue_cycle_gmres2d<R>(h, dir, batch, zero0, check, cond, s);
-    else enqueue_cycle_gmres3d<R>(h, dir, batch, zero0, check, cond, s);
+    enqueue_cycle_gmres<R>(h, dir, batch, zero0, check, cond, s);
     return;
   }
   Work<R> &W = work<R>(h);
@@ -1096,16 +1030,8 @@ void time_one(hh_handle *h, int kernel, int level, int batch, cudaStream_t s) {
   const auto om = omega<R>(h, 0);
   const bool two = h->dim == 2;
   if (kernel == 6) {   // one GMRES(m) smoothing step from a nonzero iterate
-    if (two) {
-      const Gm2dIn<R> in{W.u_post[level], W.f[level], nullptr, Lay{0, 0, 0}, ZERO_NONE};
-      enqueue_gm2d_step<R>(h, level, 0, in, W.u_pre[level], false, batch, nullptr, CHECK_NONE, 0, s);
-    } else {
-      const GmresWork<R> g = gmres_work<R>(h, level);
-      const int nb = partial_blocks_of(h, level), m = h->opt.gmres_m;
-      typename Cx<R>::T *u = W.u_post[level];
-      launch_gmres_start<R, 3>(K, u, ZERO_NONE, W.f[level], g, batch, nullptr, g.parts, nb, s);
-      launch_gmres_rest<R, 3>(K, u, ZERO_NONE, u, g, m, batch, nullptr, nb, s, h->gm_fuse);
-    }
+    const Gm2dIn<R> in{W.u_post[level], W.f[level], nullptr, Lay{0, 0, 0}, ZERO_NONE};
+    enqueue_gm_step<R>(h, level, 0, in, W.u_pre[level], false, batch, nullptr, CHECK_NONE, 0, s);
     return;
   }
   if (kernel == 4 && h->opt.smoother == HH_SMOOTH_GMRES) {   // the GMRES one-block tail
@@ -1789,11 +1715,15 @@ hh_status autotune(hh_handle *h, cudaStream_t s) {
 // whose tail (it and all coarser levels) fits kGmTailSmemMax of shared
 // memory (HH_GMTAIL=off in the environment keeps every level per-level).
 // Largest level (points per axis) of the GMRES one-block tail (HH_GMTAIL_N
-// overrides, for tuning).
-template <typename R> int gm_tail_max_n(int dim) {
+// overrides, for tuning).  A step of the many-block kernels takes 5 to 6 us on any
+// small level (complex64; 3-D 8 to 9), one of the tail about 4 us on 15^2, but the
+// tail's one SM falls behind as the points grow: the 1023^2 cycle takes 210.9 us
+// with the tail from 15^2 and 212.8 from 31^2 (255^2: 129 from 63^2, 100 from 31^2,
+// 98 from 15^2, 102 from 7^2), the 127^3 cycle 335 us from 7^3 and 393 from 15^3; in
+// complex128 (255^2, four right-hand sides) 0.73 ms from 15^2 and 0.78 from 31^2.
+int gm_tail_max_n(int dim) {
   if (const char *e = std::getenv("HH_GMTAIL_N")) return std::max(3, std::atoi(e));
-  if (dim == 3) return 15;
-  return sizeof(R) == 4 ? 31 : 15;
+  return dim == 3 ? 7 : 15;
 }
 
 template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
@@ -1808,7 +1738,7 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
     for (int l = t; l < L; ++l) N[l - t] = h->lv[l].N;
     const size_t b = h->dim == 2 ? gmres_tail_smem<R, 2>(N, L - t, h->opt.gmres_m)
                                  : gmres_tail_smem<R, 3>(N, L - t, h->opt.gmres_m);
-    if (N[0] > gm_tail_max_n<R>(h->dim)) continue;
+    if (N[0] > gm_tail_max_n(h->dim)) continue;
     if (b <= kGmTailSmemMax) { t0 = t; break; }
   }
   if (t0 < 0) return HH_OK;
@@ -1838,14 +1768,13 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
       N[i] = h->lv[l].N;
     }
     a.kbase = (int)((c * sizeof(C) + 15) / 16 * 16);
-    a.lubase = (int)((a.kbase + r * sizeof(R) + 15) / 16 * 16);
+    a.invbase = (int)((a.kbase + r * sizeof(R) + 15) / 16 * 16);
     a.smem_bytes = (int)(h->dim == 2 ? gmres_tail_smem<R, 2>(N, a.nl, a.m)
                                      : gmres_tail_smem<R, 3>(N, a.nl, a.m));
     a.f = work<R>(h).f[t0];
     a.u = work<R>(h).u_post[t0];
     a.lay = lay_of(h, t0);
-    a.lu = h->lu[dir];
-    a.piv = h->piv[dir];
+    a.inv = h->inv[dir];
     a.mm = h->m;
     if constexpr (std::is_same<R, float>::value) h->gta32[dir] = a;
     else h->gta64[dir] = a;
@@ -2011,58 +1940,32 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   h->k2c = k2_dev ? 0.0 : k2_const;
   h->fused = 0;
   if (h->opt.smoother == HH_SMOOTH_GMRES) {
-    // vectors per level, in the cycle's precision: 3-D q_0..q_3 and two of
-    // A q_j; 2-D complex128 q_0..q_2 and X q_2 (complex64 stores none)
+    // stored basis per level, in the cycle's precision: 3-D q_0..q_2, 2-D only in
+    // complex128, and complex128 X q_{m-1} as well (zero padding columns)
+    HH_CK(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device));
+    const int tb = tune_batch(h);
+    size_t parts = dim == 2 ? gm2d_max_parts(tb, h->sms) : 0;
     for (int l = 0; l + 1 < L; ++l) {
       const size_t np = (size_t)h->lv[l].S * B;
+      if (dim == 3) parts = std::max<size_t>(parts, gm3d_plan_of(h, l).blocks);
       if (h->opt.precision == HH_FP64) {
         HH_TRY(dev_alloc_n(h, &h->w64.gq[l], 4 * np));
         HH_CK(cudaMemsetAsync(h->w64.gq[l], 0, 4 * np * sizeof(double2), s));
-        if (dim == 3) {
-          HH_TRY(dev_alloc_n(h, &h->w64.gw[l], np));
-          HH_TRY(dev_alloc_n(h, &h->w64.gw2[l], np));
-          HH_CK(cudaMemsetAsync(h->w64.gw[l], 0, np * sizeof(double2), s));
-          HH_CK(cudaMemsetAsync(h->w64.gw2[l], 0, np * sizeof(double2), s));
-        }
       } else if (dim == 3) {
-        HH_TRY(dev_alloc_n(h, &h->w32.gq[l], 4 * np));
-        HH_TRY(dev_alloc_n(h, &h->w32.gw[l], np));
-        HH_TRY(dev_alloc_n(h, &h->w32.gw2[l], np));
-        HH_CK(cudaMemsetAsync(h->w32.gq[l], 0, 4 * np * sizeof(float2), s));
-        HH_CK(cudaMemsetAsync(h->w32.gw[l], 0, np * sizeof(float2), s));
-        HH_CK(cudaMemsetAsync(h->w32.gw2[l], 0, np * sizeof(float2), s));
+        HH_TRY(dev_alloc_n(h, &h->w32.gq[l], 3 * np));
+        HH_CK(cudaMemsetAsync(h->w32.gq[l], 0, 3 * np * sizeof(float2), s));
       }
     }
-    // blocks per kernel: complex64 4 per SM, enough warps to keep the
-    // stencil loads of the grid-stride loops in flight; complex128 2 per SM
-    // (bound by the FP64 pipe, where more blocks only lengthen the last
-    // block's sum over the partials); HH_GMBLOCKS overrides, for tuning
-    HH_CK(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device));
-    h->gm_cap = (h->opt.precision == HH_FP64 ? 2 : 4) * h->sms;
-    if (const char *e = std::getenv("HH_GMBLOCKS")) h->gm_cap = std::max(1, std::atoi(e));
-    HH_TRY(dev_alloc_n(h, &h->gm_parts, (size_t)h->gm_cap * kGmresParts * B));
-    // complex64: the orthogonalisation of a step and the next Arnoldi product
-    // in one kernel (fewer launches; complex128 stays unfused, since the
-    // recomputed neighbours' orthogonalisation costs FP64 operations, the
-    // bound of those kernels); HH_GMFUSE=0/1 in the environment overrides
-    h->gm_fuse = h->opt.precision != HH_FP64;
-    if (const char *e = std::getenv("HH_GMFUSE")) h->gm_fuse = std::atoi(e) != 0;
-    if (dim == 2) {
-      double *q = nullptr;   // 16 sums per block: FP64, or FP32 pairs
-      HH_TRY(dev_alloc_n(h, &q, (size_t)16 * gm2d_max_parts(tune_batch(h), h->sms) * B));
-      h->gm2_parts = q;
-      HH_TRY(dev_alloc_n(h, &h->gm2_zero, (size_t)B));
-      HH_CK(cudaMemsetAsync(h->gm2_zero, 0, (size_t)B * sizeof(int), s));
-      if (h->opt.precision == HH_FP64) {
-        HH_TRY(dev_alloc_n(h, &h->gm2_coef, (size_t)kGm2dCoef * B));
-        HH_TRY(dev_alloc_n(h, &h->gm2_parts2, (size_t)kGm2dCorr * 8 * B));
-      }
-      HH_CK(h->opt.precision == HH_FP64 ? init_gm2d<double>() : init_gm2d<float>());
+    double *q = nullptr;   // 16 sums per block: FP64, or FP32 pairs
+    HH_TRY(dev_alloc_n(h, &q, 16 * parts * B));
+    h->gm2_parts = q;
+    HH_TRY(dev_alloc_n(h, &h->gm2_zero, (size_t)B));
+    HH_CK(cudaMemsetAsync(h->gm2_zero, 0, (size_t)B * sizeof(int), s));
+    if (h->opt.precision == HH_FP64) {
+      HH_TRY(dev_alloc_n(h, &h->gm2_coef, (size_t)kGm2dCoef * B));
+      HH_TRY(dev_alloc_n(h, &h->gm2_parts2, (size_t)kGm2dCorr * 8 * B));
+      if (dim == 2) HH_CK(init_gm2d<double>());
     }
-    HH_TRY(dev_alloc_n(h, &h->gm_counter, 1));
-    HH_CK(cudaMemsetAsync(h->gm_counter, 0, sizeof(unsigned int), s));
-    HH_TRY(dev_alloc_n(h, &h->gm_gsc, (size_t)kGmresScalars * B));
-    HH_CK(cudaMemsetAsync(h->gm_gsc, 0, (size_t)kGmresScalars * B * sizeof(double), s));
   }
   if (dim == 2 && h->opt.nu1 == 1 && h->opt.nu2 == 1 && h->opt.smoother == HH_SMOOTH_JACOBI) {
     // first level whose tail (it and every coarser level) fits in shared memory
@@ -2102,8 +2005,9 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   for (int v = 0; v < kLevel0Variants; ++v)
     h->parts_cap = std::max(h->parts_cap, tile_parts(v, h->lv[0].N));
   if (dim == 3) h->parts_cap = std::max(h->parts_cap, tiles3d(h->lv[0].N));
-  if (h->gm_cap)
-    h->parts_cap = std::max(h->parts_cap, std::max(gmres_blocks(h, 0), gm2d_max_parts(tune_batch(h), h->sms)));
+  if (h->opt.smoother == HH_SMOOTH_GMRES)
+    h->parts_cap = std::max(h->parts_cap, dim == 2 ? gm2d_max_parts(tune_batch(h), h->sms)
+                                                   : gm3d_plan_of(h, 0).blocks);
   HH_TRY(dev_alloc_n(h, &h->partials, (size_t)h->parts_cap * B));
   HH_TRY(dev_alloc_n(h, &h->err, 1));
   HH_CK(cudaMemsetAsync(h->err, 0, sizeof(int), s));
@@ -2133,6 +2037,10 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     const LevelK<double> K = levelk<double>(h, L - 1, dir);
     if (dim == 2) launch_assemble_lu<2>(K, h->lu[dir], h->piv[dir], info_d + dir, s);
     else launch_assemble_lu<3>(K, h->lu[dir], h->piv[dir], info_d + dir, s);
+    if (h->opt.smoother == HH_SMOOTH_GMRES) {
+      HH_TRY(dev_alloc_n(h, &h->inv[dir], (size_t)h->m * h->m));
+      launch_invert_lu(h->lu[dir], h->piv[dir], h->m, h->inv[dir], s);
+    }
   }
   int info_h[2] = {0, 0};
   HH_CK(cudaMemcpyAsync(info_h, info_d, sizeof(info_h), cudaMemcpyDeviceToHost, s));
@@ -2169,9 +2077,9 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   // the 3-D weighted-Jacobi cycle's level-0 sweep writes one partial sum per box
   if (dim == 3 && h->opt.smoother == HH_SMOOTH_JACOBI && !pointwise3d(h))
     h->nparts = tiles3d(h->lv[0].N);
-  // the GMRES cycle's level-0 start kernel writes one partial sum per block
+  // the GMRES cycle's first level-0 step writes one partial sum per block
   if (h->opt.smoother == HH_SMOOTH_GMRES)
-    h->nparts = dim == 3 ? gmres_blocks(h, 0)
+    h->nparts = dim == 3 ? gm3d_plan_of(h, 0).blocks
                          : (h->opt.precision == HH_FP64 ? gm2d_plan_of<double>(h, 0, true)
                                                         : gm2d_plan_of<float>(h, 0, true)).blocks;
   return HH_OK;
@@ -2748,18 +2656,12 @@ int hh_cycle_kernels(const hh_handle *h) {
     return 2 * (1 + h->ngroups) + 2;
   }
   if (h->opt.smoother == HH_SMOOTH_GMRES) {
-    // 2-D: two kernels per step (complex128 three); 3-D: per level steps of 2m + 1 kernels
-    // (start, m Arnoldi products, m - 1 orthogonalisations, update; m + 2 with
-    // the fused orthogonalisation + Arnoldi kernels, m >= 2), residual +
-    // restriction, correction; then the tail (or the coarsest LU) and the
-    // stop test
-    if (h->dim == 2)
-      return (h->gtail0 > 0 ? h->gtail0 : h->L - 1) * (h->opt.precision == HH_FP64 ? 3 : 2) *
-                 (h->opt.nu1 + h->opt.nu2) + 2;
+    // per step: one basis kernel (3-D: m + 1), the update, in complex128 the
+    // coefficients between them; 3-D: residual + restriction and correction per
+    // level; then the tail (or the coarsest LU) and the stop test
     const int T = h->gtail0 > 0 ? h->gtail0 : h->L - 1;
-    const int m = h->opt.gmres_m;
-    const int step = h->gm_fuse && m >= 2 ? m + 2 : 2 * m + 1;
-    return T * ((h->opt.nu1 + h->opt.nu2) * step + 2) + 2;
+    const int step = (h->dim == 3 ? h->opt.gmres_m + 1 : 1) + (h->opt.precision == HH_FP64 ? 2 : 1);
+    return T * ((h->opt.nu1 + h->opt.nu2) * step + (h->dim == 3 ? 2 : 0)) + 2;
   }
   // per level nu1 sweeps, residual + restriction, nu2 sweeps; stop test; LU
   return (h->L - 1) * (h->opt.nu1 + 1 + h->opt.nu2) + 2;

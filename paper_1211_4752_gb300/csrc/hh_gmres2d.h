@@ -37,7 +37,7 @@ template <typename R> struct Gm2dWork {
 constexpr int kGm2dCoef = 32;   // z_0..z_2, whether a correction follows, Gram matrix (16)
 constexpr int kGm2dCorr = 128;  // blocks of the correction's sums at most
 
-template <typename R> cudaError_t init_gm2d();   // once per handle
+template <typename R> cudaError_t init_gm2d();   // once per complex128 handle
 template <typename R> Gm2dPlan gm2d_plan(int N, int m, int batch, int sms, bool restrict_);
 int gm2d_max_parts(int batch, int sms);   // blocks per right-hand side at most
 
@@ -58,7 +58,6 @@ void launch_gm2d_update(const LevelK<R> &L, typename Cx<R>::T sigma, R s, int kc
 
 template <> Gm2dPlan gm2d_plan<float>(int, int, int, int, bool);
 template <> Gm2dPlan gm2d_plan<double>(int, int, int, int, bool);
-template <> cudaError_t init_gm2d<float>();
 template <> cudaError_t init_gm2d<double>();
 template <> void launch_gm2d_basis<float>(const LevelK<float> &, float2, float, int, int,
                                           const Gm2dIn<float> &, const Gm2dWork<float> &,

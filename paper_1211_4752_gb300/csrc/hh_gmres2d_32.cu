@@ -545,8 +545,6 @@ template <> Gm2dPlan gm2d_plan<float>(int N, int m, int batch, int sms, bool res
   return p;
 }
 
-template <> cudaError_t init_gm2d<float>() { return cudaSuccess; }
-
 template <>
 void launch_gm2d_basis<float>(const LevelK<float> &L, float2 sigma, float s, int kconst, int m,
                               const Gm2dIn<float> &in, const Gm2dWork<float> &w, const Gm2dPlan &p,

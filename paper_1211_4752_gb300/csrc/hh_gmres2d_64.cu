@@ -10,6 +10,7 @@
 // 127^2 (57 to 20 per kernel chain before); the cycle of four right-hand sides at
 // 255^2 0.73 ms (1.05), of one at 1023^2 1.79 ms (2.72 with marches).
 #include "hh_gmres2d.cuh"
+#include "hh_gmres3d.h"
 
 namespace hh {
 
@@ -309,8 +310,8 @@ __device__ __forceinline__ void restrict_body(const TileCtx<R, MODE> &t, ColumnO
 // the solution (corrected seminormal equations, Bjorck 1987).
 template <int M>
 __global__ void __launch_bounds__(256)
-k_gm2d_coef(LevelK<double> L, double2 sigma, double s, Gm2dWork<double> wk, int nparts, double tol,
-            const SolveState *st) {
+k_gm2d_coef(LevelK<double> L, int rows, double2 sigma, double s, Gm2dWork<double> wk, int nparts,
+            double tol, const SolveState *st) {
   constexpr int NQP = Gram<M>::NQP;
   using A = GramAcc<double, false>;
   __shared__ double sums[8 * 16];
@@ -341,7 +342,7 @@ k_gm2d_coef(LevelK<double> L, double2 sigma, double s, Gm2dWork<double> wk, int 
   const double2 t = cscale(sigma, s);
   const double2 *q = wk.q + (size_t)b * L.S;
   const int N = L.N;
-  for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < (unsigned)(N * N); p += gridDim.x * blockDim.x) {
+  for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < (unsigned)rows * (unsigned)N; p += gridDim.x * blockDim.x) {
     const unsigned yy = p / (unsigned)N, o = yy * (unsigned)L.P + (p - yy * (unsigned)N);
     double2 v[M + 1], a[M];
 #pragma unroll
@@ -541,6 +542,18 @@ void launch_gm2d_basis<double>(const LevelK<double> &L, double2 sigma, double s,
   });
 }
 
+int launch_gm_coef(const LevelK<double> &L, int rows, double2 sigma, double s, int m,
+                   const Gm2dWork<double> &w, int nparts, int batch, const SolveState *st,
+                   cudaStream_t stream) {
+  const int nb = std::min(kGm2dCorr, (int)(((long long)rows * L.N + 1023) / 1024));
+  const double tol = gram_tol<double>(false);
+  with_m(m, [&](auto mm) {
+    launch_pdl(k_gm2d_coef<decltype(mm)::value>, dim3(nb, batch), dim3(256), 0, stream, L, rows, sigma, s,
+               w, nparts, tol, st);
+  });
+  return nb;
+}
+
 template <>
 void launch_gm2d_update<double>(const LevelK<double> &L, double2 sigma, double s, int kconst, int m,
                                 const Gm2dIn<double> &in, const Gm2dWork<double> &w, const Gm2dPlan &p,
@@ -549,8 +562,7 @@ void launch_gm2d_update<double>(const LevelK<double> &L, double2 sigma, double s
   const double tol = gram_tol<double>(false);
   with_m(m, [&](auto mm) {
     constexpr int M = decltype(mm)::value;
-    const int nb = std::min(kGm2dCorr, (L.N * L.N + 1023) / 1024);
-    launch_pdl(k_gm2d_coef<M>, dim3(nb, batch), dim3(256), 0, stream, L, sigma, s, w, p.blocks, tol, st);
+    const int nb = launch_gm_coef(L, L.N, sigma, s, M, w, p.blocks, batch, st, stream);
     // (a corrected iterate is never restricted: it belongs to the way up)
     auto go = [&](auto corr, auto rest) {
       constexpr bool CORR = decltype(corr)::value, REST = decltype(rest)::value;

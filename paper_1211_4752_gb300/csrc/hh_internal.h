@@ -138,6 +138,9 @@ void launch_finish(const SolveState *st, const double2 *src, const Lay &ls, doub
 void launch_grad_k2(const double2 *u, const double2 *lam, size_t pts,
                     int batch, double *grad, cudaStream_t s);
 
+// inverse (m x m, FP64) of the matrix whose LU factors k_assemble_lu stored
+void launch_invert_lu(const double2 *lu, const int *piv, int m, double2 *inv, cudaStream_t s);
+
 int partial_blocks(size_t pts);
 
 }  // namespace hh

@@ -214,6 +214,26 @@ int grid_cap(size_t work, int threads = 256, int cap = 8 * 152 * 4) {
 
 }  // namespace
 
+// Column j of the inverse from the LU factors (unit lower triangle, 1 / U_kk on
+// the diagonal): thread j solves for the j-th unit vector (m <= 27).
+__global__ void k_invert_lu(const double2 *lu, const int *piv, int m, double2 *inv) {
+  const int j = threadIdx.x;
+  if (j >= m) return;
+  double2 y[27];
+  for (int i = 0; i < m; ++i) {
+    y[i] = make_double2(piv[i] == j ? 1.0 : 0.0, 0.0);
+    for (int k = 0; k < i; ++k) y[i] = csub(y[i], cmul(lu[i * m + k], y[k]));
+  }
+  for (int i = m - 1; i >= 0; --i) {
+    for (int k = i + 1; k < m; ++k) y[i] = csub(y[i], cmul(lu[i * m + k], y[k]));
+    y[i] = cmul(y[i], lu[i * m + i]);
+  }
+  for (int i = 0; i < m; ++i) inv[i * m + j] = y[i];
+}
+void launch_invert_lu(const double2 *lu, const int *piv, int m, double2 *inv, cudaStream_t s) {
+  k_invert_lu<<<1, 32, 0, s>>>(lu, piv, m, inv);
+}
+
 int partial_blocks(size_t pts) { return grid_cap(pts, 256, 2 * 152); }
 
 void launch_norm2(const double2 *x, size_t stride, int batch, double *partials,

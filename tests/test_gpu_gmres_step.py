@@ -71,3 +71,35 @@ def test_krylov_space_of_one_dimension(n):
         z = mg.cycles(torch.zeros_like(g), torch.zeros_like(g), 1)   # zero residual: no correction
         assert not z.abs().max().item()
         mg.close()
+
+
+CASES_3D = [
+    # n, batch, layers, k2, form, m, nu1, nu2
+    (8, 2, 0, 20.0, "csl", 3, 1, 1),
+    (16, 1, (1, 3), ("field", 5.0, 9.0), "csl", 1, 1, 1),
+    (32, 3, (4, 2), 300.0, "csg", 2, 1, 2),
+    (64, 1, 5, ("field", 18.0, 36.0), "csl", 3, 2, 1),
+    (128, 1, 9, 60.0 ** 2, "csl", 3, 1, 1),          # plain sums
+]
+
+
+@pytest.mark.parametrize("case", CASES_3D, ids=lambda c: f"n{c[0]}-b{c[1]}-m{c[5]}-nu{c[6]}{c[7]}")
+def test_step_matches_oracle_3d(case):
+    from paper_1211_4752_gb300 import HelmholtzMG
+    n, batch, layers, k2, form, m, nu1, nu2 = case
+    if isinstance(k2, tuple):
+        k2 = W.smooth_k2(n, 3, 4, k2[1], k2[2])
+    P = int(round(math.log2(n)))
+    c = [np.exp(-1j * (math.pi / 6) / P)] * (P - 2) if form == "csg" else None
+    H = O.build_hierarchy(n, 3, k2, layers=layers, form=form, c=c, smoother="gmres", m=m, nu1=nu1, nu2=nu2)
+    kt = torch.from_numpy(k2).cuda() if isinstance(k2, np.ndarray) else k2
+    f = W.random_field((batch,) + (n - 1,) * 3, 53)
+    u0 = W.random_field(f.shape, 54, scale=1.0 / n ** 2)
+    ref = {b: O.vcycle(H, 0, u0[b], f[b]) for b in {0, batch - 1}}
+    for precision, tol in (("fp64", 1e-9), ("mixed", 1e-4)):
+        mg = HelmholtzMG(n, dim=3, k2=kt, layers=layers, form=form, c=c, smoother="gmres", gmres_m=m,
+                         nu1=nu1, nu2=nu2, precision=precision, max_batch=batch)
+        got = mg.cycles(torch.from_numpy(f).cuda(), torch.from_numpy(u0).cuda(), 1).cpu().numpy()
+        for b, r in ref.items():
+            assert np.linalg.norm(got[b] - r) <= tol * np.linalg.norm(r), (precision, b)
+        mg.close()
