@@ -157,6 +157,7 @@ struct hh_handle {
   long long fixed_kernels = 0;      // other kernels of the current solve
   long long last_kernels = -1;      // kernels of the last completed solve
   float2 *tailop[2] = {nullptr, nullptr};  // tail operator per direction (mixed)
+  double2 *tailop64[2] = {nullptr, nullptr};  // (complex128 cycles of small batches)
   int mid = 0;                      // complex64 cycles: cluster kernel for the
   int mid0 = 0, midt = 0, midcl = 0;  // levels mid0 .. midt-1 (cluster of midcl CTAs)
   float2 *tailop_mid[2] = {nullptr, nullptr};  // tail operator from level midt
@@ -633,7 +634,7 @@ void fork_check(hh_handle *h, int check, unsigned long long cond, cudaStream_t s
 }
 
 // Levels tail0 .. coarsest of a cycle: the dense tail operator where one
-// was built (complex64 cycles), else the single-block tail kernel.
+// was built (complex128: for small batches), else the single-block tail kernel.
 template <typename R>
 void enqueue_tail(hh_handle *h, int dir, int batch, const SolveState *st, cudaStream_t s) {
   if constexpr (std::is_same<R, float>::value) {
@@ -641,6 +642,14 @@ void enqueue_tail(hh_handle *h, int dir, int batch, const SolveState *st, cudaSt
       const LevelHost &v = h->lv[h->tail0];
       launch_tail_apply(h->tailop[dir], v.N, v.P, (int)v.S, h->w32.f[h->tail0],
                         h->w32.u_post[h->tail0], batch, st, s);
+      return;
+    }
+  }
+  if constexpr (std::is_same<R, double>::value) {
+    if (h->tailop64[dir] && batch <= kTailOp64Batch) {
+      const LevelHost &v = h->lv[h->tail0];
+      launch_tail_apply64(h->tailop64[dir], v.N, v.P, (int)v.S, h->w64.f[h->tail0],
+                          h->w64.u_post[h->tail0], batch, st, s);
       return;
     }
   }
@@ -1202,7 +1211,8 @@ template <typename R> hh_status tune_level(hh_handle *h, int l, cudaStream_t s, 
 // right-hand sides of level tail0 (one block each), the responses gathered
 // into rows of T and rounded to complex64.  The two N^2 x S scratch arrays
 // live only during setup.
-hh_status build_tail_op(hh_handle *h, int dir, int start, float2 **out, cudaStream_t s) {
+template <typename R>
+hh_status build_tail_op(hh_handle *h, int dir, int start, typename Cx<R>::T **out, cudaStream_t s) {
   const LevelHost &v = h->lv[start];
   const int N = v.N, P = v.P, S = (int)v.S, M = N * N;
   const size_t n = (size_t)M * S;
@@ -1220,7 +1230,7 @@ hh_status build_tail_op(hh_handle *h, int dir, int start, float2 **out, cudaStre
       a.lv[0].f = F;
       a.lv[0].u = U;
       launch_tail2d<double>(a, M, nullptr, s);
-      launch_tail_gather(U, *out, N, P, S, s);
+      launch_tail_gather<R>(U, *out, N, P, S, s);
       e = cudaStreamSynchronize(s);
       if (e == cudaSuccess) e = cudaGetLastError();
     }
@@ -1310,7 +1320,7 @@ hh_status setup_mid(hh_handle *h, cudaStream_t s) {
     if (init_mid2d<float>(cl, a.smem_bytes) != cudaSuccess) { cudaGetLastError(); continue; }
     if (mid2d_max_clusters<float>(cl, a.smem_bytes) < 1) continue;
     for (int dir = 0; dir < 2; ++dir)
-      HH_TRY(build_tail_op(h, dir, t, &h->tailop_mid[dir], s));
+      HH_TRY(build_tail_op<float>(h, dir, t, &h->tailop_mid[dir], s));
     for (int dir = 0; dir < 2; ++dir) HH_TRY(mid_layout(h, m0, t, cl, dir, &h->margs[dir]));
     h->mid = 1;
     h->mid0 = m0;
@@ -2068,7 +2078,10 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     const char *te = std::getenv("HH_TAIL");
     const bool op = !(te && std::strcmp(te, "kernel") == 0);
     if (op && h->opt.precision == HH_MIXED && h->lv[h->tail0].S <= kTailOpMaxS)
-      for (int dir = 0; dir < 2; ++dir) HH_TRY(build_tail_op(h, dir, h->tail0, &h->tailop[dir], s));
+      for (int dir = 0; dir < 2; ++dir) HH_TRY(build_tail_op<float>(h, dir, h->tail0, &h->tailop[dir], s));
+    if (op && h->opt.precision == HH_FP64 && h->lv[h->tail0].S <= kTailOpMaxS)
+      for (int dir = 0; dir < 2; ++dir)
+        HH_TRY(build_tail_op<double>(h, dir, h->tail0, &h->tailop64[dir], s));
     if (op && h->opt.precision == HH_MIXED) HH_TRY(setup_mid(h, s));
     HH_TRY(autotune(h, s));
     if (op) HH_TRY(setup_persist(h, s));

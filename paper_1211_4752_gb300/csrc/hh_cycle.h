@@ -305,7 +305,13 @@ void launch_tail_list(const TailList &a, int blocks, cudaStream_t s);
 void launch_check_list(const CheckList &a, cudaStream_t s);
 
 void launch_unit_rhs(double2 *F, int N, int P, int S, cudaStream_t s);
-void launch_tail_gather(const double2 *U, float2 *T, int N, int P, int S, cudaStream_t s);
+template <typename R>
+void launch_tail_gather(const double2 *U, typename Cx<R>::T *T, int N, int P, int S, cudaStream_t s);
+// complex128 tail operator, for batches of at most kTailOp64Batch right-hand sides:
+// 7.5 us each, against 60 us for the tail kernel whatever the batch
+constexpr int kTailOp64Batch = 6;
+void launch_tail_apply64(const double2 *T, int N, int P, int S, const double2 *f, double2 *u,
+                         int batch, const SolveState *st, cudaStream_t s);
 void launch_tail_apply(const float2 *T, int N, int P, int S, const float2 *f, float2 *u,
                        int batch, const SolveState *st, cudaStream_t s);
 

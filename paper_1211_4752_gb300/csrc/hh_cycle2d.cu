@@ -230,19 +230,20 @@ __global__ void k_unit_rhs(double2 *F, int N, int P, int S) {
 }
 
 // T[i * S + pos(j)] = U[j * S + pos(i)]: response at point i to a unit
-// right-hand side at point j, rounded to complex64; padding columns zero.
-__global__ void k_tail_gather(const double2 *U, float2 *T, int N, int P, int S) {
+// right-hand side at point j, in the cycle's precision; padding columns zero.
+template <typename R>
+__global__ void k_tail_gather(const double2 *U, typename Cx<R>::T *T, int N, int P, int S) {
   const int M = N * N;
   const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= (size_t)M * S) return;
   const int i = (int)(q / S), c = (int)(q - (size_t)i * S);
   const int cy = c / P, cx = c - cy * P;
-  float2 t = make_float2(0.f, 0.f);
+  typename Cx<R>::T t = czero<typename Cx<R>::T>();
   if (cx < N) {
     const int j = cy * N + cx;
     const int iy = i / N, ix = i - iy * N;
     const double2 v = U[(size_t)j * S + iy * P + ix];
-    t = make_float2((float)v.x, (float)v.y);
+    t = cmk((R)v.x, (R)v.y);
   }
   T[q] = t;
 }
@@ -305,15 +306,68 @@ __global__ void __launch_bounds__(256) k_tail_apply(const float2 *__restrict__ T
   }
 }
 
+// The same product in complex128, one right-hand side after the other: a warp per
+// row of T (its loads issued before the dependency wait), f staged in shared
+// memory.  Bound by the FP64 pipe: 961 x 961 complex products take 7 us on the
+// whole chip; the levels' own kernel (k_tail2d) runs them on one SM per
+// right-hand side, 60 us for any batch up to the number of SMs.
+constexpr int kTailRows64 = 7;   // warps (rows) per block: 138 blocks for 31^2
+__global__ void __launch_bounds__(32 * kTailRows64)
+k_tail_apply64(const double2 *__restrict__ T, int N, int P, int S, const double2 *__restrict__ f,
+               double2 *__restrict__ u, int batch, const SolveState *st) {
+  constexpr int Q = kTailOpMaxS / 32;
+  __shared__ double2 sf[kTailOpMaxS];
+  const int i = blockIdx.x * kTailRows64 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const bool row = i < N * N;
+  double2 t[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int c = lane + 32 * q;
+    t[q] = row && c < S ? __ldg(T + (size_t)i * S + c) : make_double2(0.0, 0.0);
+  }
+  griddep_wait();
+  griddep_launch_dependents();
+  for (int b = 0; b < batch; ++b) {
+    if (!__syncthreads_and(!(st && !st[b].active))) continue;   // block-uniform
+    for (int c = threadIdx.x; c < kTailOpMaxS; c += 32 * kTailRows64)
+      sf[c] = c < S && (c & (P - 1)) < N ? f[(size_t)b * S + c] : make_double2(0.0, 0.0);
+    __syncthreads();
+    double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const double2 v = sf[lane + 32 * q];
+      ax = fma(t[q].x, v.x, ax);
+      bx = fma(-t[q].y, v.y, bx);
+      ay = fma(t[q].x, v.y, ay);
+      by = fma(t[q].y, v.x, by);
+    }
+    ax += bx;
+    ay += by;
+    for (int o = 16; o > 0; o >>= 1) {
+      ax += __shfl_xor_sync(0xffffffffu, ax, o);
+      ay += __shfl_xor_sync(0xffffffffu, ay, o);
+    }
+    if (row && lane == 0) u[(size_t)b * S + (i / N) * P + i % N] = make_double2(ax, ay);
+  }
+}
+
 }  // namespace
 
 void launch_unit_rhs(double2 *F, int N, int P, int S, cudaStream_t s) {
   const int M = N * N;
   k_unit_rhs<<<(M + 255) / 256, 256, 0, s>>>(F, N, P, S);
 }
-void launch_tail_gather(const double2 *U, float2 *T, int N, int P, int S, cudaStream_t s) {
+template <typename R>
+void launch_tail_gather(const double2 *U, typename Cx<R>::T *T, int N, int P, int S, cudaStream_t s) {
   const size_t tot = (size_t)N * N * S;
-  k_tail_gather<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(U, T, N, P, S);
+  k_tail_gather<R><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(U, T, N, P, S);
+}
+template void launch_tail_gather<float>(const double2 *, float2 *, int, int, int, cudaStream_t);
+template void launch_tail_gather<double>(const double2 *, double2 *, int, int, int, cudaStream_t);
+void launch_tail_apply64(const double2 *T, int N, int P, int S, const double2 *f, double2 *u,
+                         int batch, const SolveState *st, cudaStream_t s) {
+  launch_pdl(k_tail_apply64, dim3((N * N + kTailRows64 - 1) / kTailRows64), dim3(32 * kTailRows64), 0, s,
+             T, N, P, S, f, u, batch, st);
 }
 void launch_tail_apply(const float2 *T, int N, int P, int S, const float2 *f, float2 *u,
                        int batch, const SolveState *st, cudaStream_t s) {
