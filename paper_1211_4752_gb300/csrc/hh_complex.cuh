@@ -55,4 +55,23 @@ template <typename C> __device__ __forceinline__ C crcp(C b) {
   return cmk(b.x * s, -b.y * s);
 }
 
+// c - a b
+template <typename C> __device__ __forceinline__ C cfnma(C a, C b, C c) {
+  return cmk(c.x - a.x * b.x + a.y * b.y, c.y - a.x * b.y - a.y * b.x);
+}
+// d - beta k2 (beta is real on the finest level)
+template <typename C, typename R> __device__ __forceinline__ C diag_less(C d, C beta, R k2) {
+  d.x = fmaf_any(-beta.x, k2, d.x);
+  if (beta.y != R(0)) d.y = fmaf_any(-beta.y, k2, d.y);
+  return d;
+}
+// omega / D: one real division (omega is real in all but the ablation)
+template <typename C> __device__ __forceinline__ C jacobi_weight(C omega, C D) {
+  if (omega.y == decltype(D.x)(0)) {
+    const auto s = omega.x / (D.x * D.x + D.y * D.y);
+    return cmk(D.x * s, -D.y * s);
+  }
+  return cmul(omega, crcp(D));
+}
+
 }  // namespace hh

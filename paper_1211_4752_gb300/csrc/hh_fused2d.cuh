@@ -164,6 +164,26 @@ __device__ __forceinline__ C resid_uniform(C fv, C vc, C sn, C c0, C Dk) {
   return r;
 }
 
+// The same where c_0, D_k and W_k are real (the finest level's uniform tiles: no
+// shift, a real weight; wk, dk their real parts): 4 + 2 multiply-adds instead of
+// 8 + 4.  The dropped terms are products with zero: the results are the same.  And
+// from a zero iterate (every coarse level's pre-smoothing) v = W_k f.  Both count in
+// complex128, whose kernels are bound by the FP64 pipe.  Measured with the weight made
+// on the host (LevelK::wk): a 1023^2 down pass 143 -> 115 us, up pass 87 -> 80, 511^2
+// 50 -> 46 and 35 -> 25; per point about 50 and 35 FP64 instructions, which at the
+// pipe's 64 cycles per warp take 85 % of the time.
+template <typename C, typename R>
+__device__ __forceinline__ void jacobi_real(C fv, C uc, C sn, R c0, R dk, R wk, C &r, C &v) {
+  r.x = fmaf_any(-dk, uc.x, fmaf_any(c0, sn.x, fv.x));
+  r.y = fmaf_any(-dk, uc.y, fmaf_any(c0, sn.y, fv.y));
+  v.x = fmaf_any(wk, r.x, uc.x);
+  v.y = fmaf_any(wk, r.y, uc.y);
+}
+template <typename C, typename R>
+__device__ __forceinline__ C resid_real(C fv, C vc, C sn, R c0, R dk) {
+  return cmk(fmaf_any(-dk, vc.x, fmaf_any(c0, sn.x, fv.x)), fmaf_any(-dk, vc.y, fmaf_any(c0, sn.y, fv.y)));
+}
+
 // Two complex64 values (a column pair) as one 16-byte shared/global access.
 __device__ __forceinline__ float2 lo2(float4 q) { return make_float2(q.x, q.y); }
 __device__ __forceinline__ float2 hi2(float4 q) { return make_float2(q.z, q.w); }
@@ -287,8 +307,10 @@ __device__ __forceinline__ void down_compute(
   // D = 4 c0 - beta k2, W = omega / D
   const C c0 = FAST ? L.c0 : zc;
   const C d0 = FAST ? cscale(c0, R(4)) : zc;
-  const C Dk = FAST ? csub(d0, cscale(L.beta, kc)) : zc;
-  const C Wk = FAST ? cmul(omega, crcp(Dk)) : zc;
+  const C Dk = FAST ? L.dk : zc, Wk = FAST ? L.wk : zc;
+  // every coefficient real (with constant k: D_k and W_k too); complex64's uniform
+  // tiles of constant k take the paired path
+  const bool real = FAST && sizeof(R) == 8 && c0.y == R(0) && L.beta.y == R(0) && omega.y == R(0);
 
   // v = u + omega D^{-1}(f - A u) on tile + 1; |f - A u|^2 on the tile.
   if constexpr (PAIRS) {
@@ -332,26 +354,31 @@ __device__ __forceinline__ void down_compute(
           if (in) {
             const C fv = fcol[k * FW];
             C r;
-            if (FAST && kconst) {
+            if (FAST && kconst && zero) {
+              r = fv;
+              v = real ? cscale(fv, Wk.x) : cmul(Wk, fv);
+            } else if (FAST && kconst && real) {
+              jacobi_real(fv, uc, cadd(cadd(ul, ur), cadd(un, ud)), c0.x, Dk.x, Wk.x, r, v);
+            } else if (FAST && kconst) {
               jacobi_uniform(fv, uc, cadd(cadd(ul, ur), cadd(un, ud)), c0, Dk, Wk, r, v);
+            } else if (FAST && real) {
+              const R dk = fmaf_any(-L.beta.x, kcol[k * KW], d0.x);
+              jacobi_real(fv, uc, cadd(cadd(ul, ur), cadd(un, ud)), c0.x, dk, omega.x / dk, r, v);
             } else {
               const R kk = kconst ? kc : kcol[k * KW];
-              const C D = FAST ? csub(d0, cscale(L.beta, kk))
-                               : csub(cadd(cdg, s_cy[VH + ty]), cscale(L.beta, kk));
-              const C Wd = cmul(omega, crcp(D));
+              const C D = diag_less(FAST ? d0 : cadd(cdg, s_cy[VH + ty]), L.beta, kk);
               r = fv;
               if (!zero) {
-                C nb;
-                if (FAST) nb = cmul(c0, cadd(cadd(ul, ur), cadd(un, ud)));
+                if (FAST) r = cfma(c0, cadd(cadd(ul, ur), cadd(un, ud)), r);
                 else {
-                  nb = cmul(clo, ul);
-                  nb = cfma(cup, ur, nb);
-                  nb = cfma(s_cy[ty], un, nb);
-                  nb = cfma(s_cy[2 * VH + ty], ud, nb);
+                  r = cfma(clo, ul, r);
+                  r = cfma(cup, ur, r);
+                  r = cfma(s_cy[ty], un, r);
+                  r = cfma(s_cy[2 * VH + ty], ud, r);
                 }
-                r = cadd(csub(r, cmul(D, uc)), nb);
+                r = cfnma(D, uc, r);
               }
-              v = cadd(uc, cmul(Wd, r));
+              v = cfma(jacobi_weight(omega, D), r, uc);
             }
             if (colown && ty >= 1 && ty <= BY) {
               vo[k * P] = v;
@@ -396,23 +423,24 @@ __device__ __forceinline__ void down_compute(
           C r = zc;
           if (colin && (!CHECK || y0 + ry < N)) {
             const C fv = fcol[k * FW];
-            if (FAST && kconst) {
+            if (FAST && real) {
+              const R dk = kconst ? Dk.x : fmaf_any(-L.beta.x, kcol[k * KW], d0.x);
+              r = resid_real(fv, vc, cadd(cadd(vl, vr), cadd(vn, vd)), c0.x, dk);
+            } else if (FAST && kconst) {
               r = resid_uniform(fv, vc, cadd(cadd(vl, vr), cadd(vn, vd)), c0, Dk);
             } else {
               const int ty = ry + 1;
-              C D, nb;
               const R kk = kconst ? kc : kcol[k * KW];
+              const C D = diag_less(FAST ? d0 : cadd(cdg, s_cy[VH + ty]), L.beta, kk);
+              r = cfnma(D, vc, fv);
               if (FAST) {
-                D = csub(d0, cscale(L.beta, kk));
-                nb = cmul(c0, cadd(cadd(vl, vr), cadd(vn, vd)));
+                r = cfma(c0, cadd(cadd(vl, vr), cadd(vn, vd)), r);
               } else {
-                D = csub(cadd(cdg, s_cy[VH + ty]), cscale(L.beta, kk));
-                nb = cmul(clo, vl);
-                nb = cfma(cup, vr, nb);
-                nb = cfma(s_cy[ty], vn, nb);
-                nb = cfma(s_cy[2 * VH + ty], vd, nb);
+                r = cfma(clo, vl, r);
+                r = cfma(cup, vr, r);
+                r = cfma(s_cy[ty], vn, r);
+                r = cfma(s_cy[2 * VH + ty], vd, r);
               }
-              r = cadd(csub(fv, cmul(D, vc)), nb);
             }
           }
           rcol[k * SRW] = r;
@@ -652,8 +680,8 @@ __device__ __forceinline__ void up_compute(const LevelK<R> &L, typename Cx<R>::T
   // u' = w + omega D^{-1}(f - A w) on the tile (column segments of RS rows)
   const C c0 = FAST ? L.c0 : zc;
   const C d0 = FAST ? cscale(c0, R(4)) : zc;
-  const C Dk = FAST ? csub(d0, cscale(L.beta, kc)) : zc;
-  const C Wk = FAST ? cmul(omega, crcp(Dk)) : zc;
+  const C Dk = FAST ? L.dk : zc, Wk = FAST ? L.wk : zc;
+  const bool real = FAST && sizeof(R) == 8 && c0.y == R(0) && L.beta.y == R(0) && omega.y == R(0);
   if constexpr (PAIRS) {
     up_u_pairs<BX, BY>(s_w, s_f, ob, P, x0, y0, c0, Dk, Wk);
   } else {
@@ -680,27 +708,28 @@ __device__ __forceinline__ void up_compute(const LevelK<R> &L, typename Cx<R>::T
           if (colin && (!CHECK || y0 + ly < N)) {
             const C fv = fcol[k * BX];
             C u;
-            if (FAST && kconst) {
+            if (FAST && real) {
+              const R dk = kconst ? Dk.x : fmaf_any(-L.beta.x, kcol[k * BX], d0.x);
+              const R wk = kconst ? Wk.x : omega.x / dk;
+              C r;
+              jacobi_real(fv, wc, cadd(cadd(wl, wr), cadd(wn, wd)), c0.x, dk, wk, r, u);
+            } else if (FAST && kconst) {
               C r;
               jacobi_uniform(fv, wc, cadd(cadd(wl, wr), cadd(wn, wd)), c0, Dk, Wk, r, u);
             } else {
-              C D, Wd, nb;
               const R kk = kconst ? kc : kcol[k * BX];
+              const int ty = ly + 1;
+              const C D = diag_less(FAST ? d0 : cadd(cdg, s_cy[WH + ty]), L.beta, kk);
+              C r = cfnma(D, wc, fv);
               if (FAST) {
-                D = csub(d0, cscale(L.beta, kk));
-                Wd = cmul(omega, crcp(D));
-                nb = cmul(c0, cadd(cadd(wl, wr), cadd(wn, wd)));
+                r = cfma(c0, cadd(cadd(wl, wr), cadd(wn, wd)), r);
               } else {
-                const int ty = ly + 1;
-                D = csub(cadd(cdg, s_cy[WH + ty]), cscale(L.beta, kk));
-                Wd = cmul(omega, crcp(D));
-                nb = cmul(clo, wl);
-                nb = cfma(cup, wr, nb);
-                nb = cfma(s_cy[ty], wn, nb);
-                nb = cfma(s_cy[2 * WH + ty], wd, nb);
+                r = cfma(clo, wl, r);
+                r = cfma(cup, wr, r);
+                r = cfma(s_cy[ty], wn, r);
+                r = cfma(s_cy[2 * WH + ty], wd, r);
               }
-              const C r = cadd(csub(fv, cmul(D, wc)), nb);
-              u = cadd(wc, cmul(Wd, r));
+              u = cfma(jacobi_weight(omega, D), r, wc);
             }
             oo[k * P] = u;
           }

@@ -34,6 +34,8 @@ template <typename R> struct LevelK {
   int ulo, uhi;    // nodes ulo..uhi (every axis) have lo = up = c0, dg = 2 c0
   C c0;            // (the uniform region away from ECS layers); ulo > uhi: none
   R kc;            // k^2 where it is constant (k2 then holds kc everywhere)
+  int kconst;      // whether it is
+  C dk, wk;        // then: the uniform region's diagonal 2 dim c0 - beta kc, and omega / dk
 };
 
 // Layout of an array of another level (e.g. the coarse one of a transfer).
