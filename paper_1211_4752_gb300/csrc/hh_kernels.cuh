@@ -525,7 +525,7 @@ void launch_inject(const double *kf, const Lay &lf, double *kc, const Lay &lc,
   k_inject<DIM><<<grid_for(npts<DIM>(lc.N)), 256, 0, s>>>(kf, lf, kc, lc);
 }
 
-#define HH_INSTANTIATE_DIM(DIM)                                                \
+#define HH_INSTANTIATE_POINTWISE(DIM)                                          \
   template void launch_smooth<float, DIM>(                                     \
       const LevelK<float> &, const float2 *, int, const float2 *, float2 *,    \
       float2, int, const SolveState *, double *, int, cudaStream_t);           \
@@ -551,7 +551,9 @@ void launch_inject(const double *kf, const Lay &lf, double *kc, const Lay &lc,
                                          cudaStream_t);                        \
   template void launch_apply<double, DIM>(const LevelK<double> &,              \
                                           const double2 *, double2 *, int,     \
-                                          cudaStream_t);                       \
+                                          cudaStream_t);
+
+#define HH_INSTANTIATE_DIM(DIM)                                                \
   template void launch_refine<DIM>(const LevelK<double> &, const double2 *,    \
                                    int, const float2 *, double2 *,             \
                                    const double2 *, float2 *, int,             \

@@ -51,6 +51,27 @@ def close(got, ref, tol):
 
 
 @pytest.mark.parametrize("case", CASES, ids=lambda c: f"n{c[0]}-b{c[1]}-{c[4]}")
+def test_steps_match_oracle(case):
+    H, mg = make(case)
+    Ha = O.adjoint_hierarchy(H)
+    B = case[1]
+    for l in range(min(3, len(H.levels) - 1)):
+        lv, lc = H.levels[l], H.levels[l + 1]
+        u, f = (W.random_field((B,) + lv.shape, 61 + i) for i in range(2))
+        e = W.random_field((B,) + lc.shape, 63)
+        for adj, hier in ((False, H), (True, Ha)):
+            ref = np.stack([O.apply_operator(hier.levels[l], x) for x in u])
+            assert close(mg.apply(dev(u), level=l, adjoint=adj), ref, 1e-13), (l, adj)
+        ref = np.stack([O.jacobi(lv, u[b], f[b], H.omega) for b in range(B)])
+        assert close(mg.smooth(l, dev(u), dev(f)), ref, 1e-13), l
+        ref = np.stack([H.c[l] * O.restrict_fw(f[b] - O.apply_operator(lv, u[b])) for b in range(B)])
+        assert close(mg.residual_restrict(l, dev(u), dev(f)), ref, 1e-12), l
+        ref = np.stack([O.jacobi(lv, u[b] + O.prolong(e[b]), f[b], H.omega) for b in range(B)])
+        assert close(mg.correct_smooth(l, dev(u), dev(e), dev(f)), ref, 1e-13), l
+    mg.close()
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"n{c[0]}-b{c[1]}-{c[4]}")
 def test_complex128_cycles_match_oracle(case):
     """Two cycles from zero (the passes' zero branch) and from an iterate; the batch
     of 7 runs the tail levels' own kernel, the others the dense operator."""
