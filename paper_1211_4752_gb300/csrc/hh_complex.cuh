@@ -59,19 +59,39 @@ template <typename C> __device__ __forceinline__ C crcp(C b) {
 template <typename C> __device__ __forceinline__ C cfnma(C a, C b, C c) {
   return cmk(c.x - a.x * b.x + a.y * b.y, c.y - a.x * b.y - a.y * b.x);
 }
-// d - beta k2 (beta is real on the finest level)
+// d - beta k2.  In complex128 a uniform branch leaves out the imaginary part of a real
+// beta (the finest level's); in complex64 a branch costs more than it saves.
 template <typename C, typename R> __device__ __forceinline__ C diag_less(C d, C beta, R k2) {
   d.x = fmaf_any(-beta.x, k2, d.x);
-  if (beta.y != R(0)) d.y = fmaf_any(-beta.y, k2, d.y);
+  if (sizeof(R) == 4 || beta.y != R(0)) d.y = fmaf_any(-beta.y, k2, d.y);
   return d;
 }
 // omega / D: one real division (omega is real in all but the ablation)
 template <typename C> __device__ __forceinline__ C jacobi_weight(C omega, C D) {
-  if (omega.y == decltype(D.x)(0)) {
+  if (sizeof(D.x) == 8 && omega.y == decltype(D.x)(0)) {
     const auto s = omega.x / (D.x * D.x + D.y * D.y);
     return cmk(D.x * s, -D.y * s);
   }
   return cmul(omega, crcp(D));
+}
+
+// f - (D u - the neighbours' part) of a 5-point row with its own coefficients.
+// complex128 counts FP64 instructions: one chain of multiply-adds; complex64, whose
+// small levels wait for the chain, two shorter ones and an addition.
+template <typename C>
+__device__ __forceinline__ C resid_row(C f, C D, C u, C lx, C uw, C ux, C ue, C ly, C un, C uy, C us) {
+  if (sizeof(f.x) == 8) {
+    C r = cfnma(D, u, f);
+    r = cfma(lx, uw, r);
+    r = cfma(ux, ue, r);
+    r = cfma(ly, un, r);
+    return cfma(uy, us, r);
+  }
+  C nb = cmul(lx, uw);
+  nb = cfma(ux, ue, nb);
+  nb = cfma(ly, un, nb);
+  nb = cfma(uy, us, nb);
+  return cadd(csub(f, cmul(D, u)), nb);
 }
 
 }  // namespace hh

@@ -369,14 +369,8 @@ __device__ __forceinline__ void down_compute(
               const C D = diag_less(FAST ? d0 : cadd(cdg, s_cy[VH + ty]), L.beta, kk);
               r = fv;
               if (!zero) {
-                if (FAST) r = cfma(c0, cadd(cadd(ul, ur), cadd(un, ud)), r);
-                else {
-                  r = cfma(clo, ul, r);
-                  r = cfma(cup, ur, r);
-                  r = cfma(s_cy[ty], un, r);
-                  r = cfma(s_cy[2 * VH + ty], ud, r);
-                }
-                r = cfnma(D, uc, r);
+                if (FAST) r = cfnma(D, uc, cfma(c0, cadd(cadd(ul, ur), cadd(un, ud)), r));
+                else r = resid_row(r, D, uc, clo, ul, cup, ur, s_cy[ty], un, s_cy[2 * VH + ty], ud);
               }
               v = cfma(jacobi_weight(omega, D), r, uc);
             }
@@ -432,15 +426,8 @@ __device__ __forceinline__ void down_compute(
               const int ty = ry + 1;
               const R kk = kconst ? kc : kcol[k * KW];
               const C D = diag_less(FAST ? d0 : cadd(cdg, s_cy[VH + ty]), L.beta, kk);
-              r = cfnma(D, vc, fv);
-              if (FAST) {
-                r = cfma(c0, cadd(cadd(vl, vr), cadd(vn, vd)), r);
-              } else {
-                r = cfma(clo, vl, r);
-                r = cfma(cup, vr, r);
-                r = cfma(s_cy[ty], vn, r);
-                r = cfma(s_cy[2 * VH + ty], vd, r);
-              }
+              if (FAST) r = cfnma(D, vc, cfma(c0, cadd(cadd(vl, vr), cadd(vn, vd)), fv));
+              else r = resid_row(fv, D, vc, clo, vl, cup, vr, s_cy[ty], vn, s_cy[2 * VH + ty], vd);
             }
           }
           rcol[k * SRW] = r;
@@ -720,15 +707,9 @@ __device__ __forceinline__ void up_compute(const LevelK<R> &L, typename Cx<R>::T
               const R kk = kconst ? kc : kcol[k * BX];
               const int ty = ly + 1;
               const C D = diag_less(FAST ? d0 : cadd(cdg, s_cy[WH + ty]), L.beta, kk);
-              C r = cfnma(D, wc, fv);
-              if (FAST) {
-                r = cfma(c0, cadd(cadd(wl, wr), cadd(wn, wd)), r);
-              } else {
-                r = cfma(clo, wl, r);
-                r = cfma(cup, wr, r);
-                r = cfma(s_cy[ty], wn, r);
-                r = cfma(s_cy[2 * WH + ty], wd, r);
-              }
+              C r;
+              if (FAST) r = cfnma(D, wc, cfma(c0, cadd(cadd(wl, wr), cadd(wn, wd)), fv));
+              else r = resid_row(fv, D, wc, clo, wl, cup, wr, s_cy[ty], wn, s_cy[2 * WH + ty], wd);
               u = cfma(jacobi_weight(omega, D), r, wc);
             }
             oo[k * P] = u;

@@ -134,11 +134,7 @@ __device__ __forceinline__ void walk_rows(const Walk2dArgs<R> &A, int b, bool ze
         r = cfnma(lo, vm, r);
         r = cfnma(up, vp, r);
       } else {
-        r = cfnma(D, v, fv);
-        r = cfma(lox, vw, r);
-        r = cfma(upx, ve, r);
-        r = cfma(lo, vm, r);
-        r = cfma(up, vp, r);
+        r = resid_row(fv, D, v, lox, vw, upx, ve, lo, vm, up, vp);
       }
     }
     if (KIND == APPLY) {
