@@ -169,9 +169,9 @@ __device__ __forceinline__ C resid_uniform(C fv, C vc, C sn, C c0, C Dk) {
 // 8 + 4.  The dropped terms are products with zero: the results are the same.  And
 // from a zero iterate (every coarse level's pre-smoothing) v = W_k f.  Both count in
 // complex128, whose kernels are bound by the FP64 pipe.  Measured with the weight made
-// on the host (LevelK::wk): a 1023^2 down pass 143 -> 115 us, up pass 87 -> 80, 511^2
-// 50 -> 46 and 35 -> 25; per point about 50 and 35 FP64 instructions, which at the
-// pipe's 64 cycles per warp take 85 % of the time.
+// on the host (LevelK::wk) and three blocks per SM: a 1023^2 down pass 143 -> 115-121 us,
+// up pass 87 -> 74, 511^2 50 -> 44 and 35 -> 24; per point about 50 and 35 FP64
+// instructions, which at the pipe's 64 cycles per warp take 85 to 90 % of the time.
 template <typename C, typename R>
 __device__ __forceinline__ void jacobi_real(C fv, C uc, C sn, R c0, R dk, R wk, C &r, C &v) {
   r.x = fmaf_any(-dk, uc.x, fmaf_any(c0, sn.x, fv.x));
@@ -552,8 +552,10 @@ __device__ __forceinline__ void down_pass_tile(
   }
 }
 
+// (Blocks per SM: six in complex64, from 40 registers; three in complex128, from 80:
+// with 95 and two blocks the 1023^2 cycle took 322 us instead of 310.)
 template <typename R, int BX, int BY>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 1)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 3)
 k_down2d(const __grid_constant__ DownMaps maps, LevelK<R> L, int zero_mode,
          typename Cx<R>::T *__restrict__ v_out, typename Cx<R>::T *__restrict__ fc,
          typename Cx<R>::T cs, typename Cx<R>::T omega, int kconst, Lay lc,
@@ -790,7 +792,7 @@ __device__ __forceinline__ void up_pass_tile(const UpMaps &maps, const LevelK<R>
 }
 
 template <typename R, int BX, int BY>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 1)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 3)
 k_up2d(const __grid_constant__ UpMaps maps, LevelK<R> L, typename Cx<R>::T *__restrict__ u_out,
        typename Cx<R>::T omega, int kconst, const SolveState *__restrict__ st, int *err) {
   up_pass_tile<R, BX, BY>(maps, L, u_out, omega, kconst, st, err, blockIdx.x, blockIdx.y,
