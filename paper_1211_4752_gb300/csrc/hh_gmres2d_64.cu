@@ -5,10 +5,11 @@
 // small: a block works on tiles of 56 columns and up to 32 rows in shared memory,
 // a thread per column and run of rows, the values above and below carried in
 // registers.  Small levels: a thread per point of 8 x 8 tiles (hh_gmres2d.cuh).
-// Measured (GB300): a GMRES(3) step takes 434 us at 1023^2 (446 with a kernel and a
-// reduction per Arnoldi step, 669 with marches), 145 at 511^2, 60 at 255^2, 40 at
-// 127^2 (57 to 20 per kernel chain before); the cycle of four right-hand sides at
-// 255^2 0.73 ms (1.05), of one at 1023^2 1.79 ms (2.72 with marches).
+// Measured (GB300; in brackets a kernel and a reduction per Arnoldi step): a GMRES(3)
+// step takes 412 us at 1023^2 (393; with marches 669), 139 at 511^2 (139), 59 at
+// 255^2 (75), 40 at 127^2 (50) and 21 at 63^2 (48), and of four right-hand sides at
+// 1023^2 1204 (1420); the cycle of one at 1023^2 1.71 ms (1.98), of four there 4.58
+// (5.49) and at 255^2 0.71 (1.05).
 #include "hh_gmres2d.cuh"
 #include "hh_gmres3d.h"
 
@@ -22,7 +23,7 @@ namespace {
 template <typename R, int MODE> struct ColumnOp {
   using C = typename Cx<R>::T;
   C c0, D0, sb, sd;        // uniform: c_0, 4 c_0, s beta, s (4 c_0 - sigma)
-  C lo, up, dg, sigma, beta;
+  C lo, up, dg, dgs, sigma, beta;   // dgs = dg - sigma
   R cf, s, kc;
   __device__ __forceinline__ ColumnOp(const LevelK<R> &L, C sigma_, R s_)
       : sigma(sigma_), beta(L.beta), s(s_), kc(L.kc) {
@@ -39,6 +40,7 @@ template <typename R, int MODE> struct ColumnOp {
     const bool in = (unsigned)x < (unsigned)L.N;
     lo = in ? L.coef[x] : czero<C>();
     dg = in ? L.coef[L.N + x] : czero<C>();
+    dgs = csub(dg, sigma);
     up = in ? L.coef[2 * L.N + x] : czero<C>();
   }
   __device__ __forceinline__ C neighbours(const C *rc, C vw, C ve, C vn, C vs) const {
@@ -50,31 +52,38 @@ template <typename R, int MODE> struct ColumnOp {
   // X v = s (A - sigma) v; rc: the row's coefficients, kv: k^2 of the point
   __device__ __forceinline__ C X(C v, C vw, C ve, C vn, C vs, const C *rc, R kv) const {
     if (MODE == GENERAL) {
-      const C d = csub(csub(cadd(dg, rc[1]), sigma), cscale(beta, kv));
+      const C d = diag_less(cadd(dgs, rc[1]), beta, kv);
       return cscale(csub(cmul(d, v), neighbours(rc, vw, ve, vn, vs)), s);
     }
     const C sn = cadd(cadd(vw, ve), cadd(vn, vs));
     C r = cmk(-cf * sn.x, -cf * sn.y);
     if (MODE == UNIFORM) {
-      C d;
-      d.x = fmaf_any(-sb.x, kv, sd.x);
-      d.y = fmaf_any(-sb.y, kv, sd.y);
-      r = cfma(d, v, r);
+      // (beta and sigma are real on the finest level: uniform branches leave out
+      // the products with zero here and below)
+      const R dx = fmaf_any(-sb.x, kv, sd.x);
+      r = cmk(fmaf_any(dx, v.x, r.x), fmaf_any(dx, v.y, r.y));
+      if (beta.y != R(0)) {
+        const R dy = fmaf_any(-sb.y, kv, sd.y);
+        r = cmk(fmaf_any(-dy, v.y, r.x), fmaf_any(dy, v.x, r.y));
+      }
     }
     return r;
   }
   __device__ __forceinline__ C resid(C f, C v, C vw, C ve, C vn, C vs, const C *rc, R kv) const {
     if (MODE == GENERAL) {
-      const C d = csub(cadd(dg, rc[1]), cscale(beta, kv));
-      return cadd(csub(f, cmul(d, v)), neighbours(rc, vw, ve, vn, vs));
+      const C d = diag_less(cadd(dg, rc[1]), beta, kv);
+      return resid_row(f, d, v, lo, vw, up, ve, rc[0], vn, rc[2], vs);
     }
     const C sn = cadd(cadd(vw, ve), cadd(vn, vs));
     const R kk = MODE == UNIFORM_K ? kc : kv;
-    C d, r;
-    d.x = fmaf_any(-beta.x, kk, D0.x);
-    d.y = -beta.y * kk;
-    r.x = fmaf_any(c0.x, sn.x, fmaf_any(-d.x, v.x, fmaf_any(d.y, v.y, f.x)));
-    r.y = fmaf_any(c0.x, sn.y, fmaf_any(-d.x, v.y, fmaf_any(-d.y, v.x, f.y)));
+    const R dx = fmaf_any(-beta.x, kk, D0.x);
+    C r;
+    r.x = fmaf_any(c0.x, sn.x, fmaf_any(-dx, v.x, f.x));
+    r.y = fmaf_any(c0.x, sn.y, fmaf_any(-dx, v.y, f.y));
+    if (beta.y != R(0)) {
+      const R dy = beta.y * kk;
+      r = cmk(fmaf_any(-dy, v.y, r.x), fmaf_any(dy, v.x, r.y));
+    }
     return r;
   }
 };
@@ -185,7 +194,7 @@ __device__ __forceinline__ void tile_vectors(const TileCtx<R, MODE> &t, ColumnOp
   }
   if (M >= 3 && last >= 2) {
     t.template walk<TX + XH - 6, false>(op, A, 3, H - 6, [](int, int, int) { return C(); },
-                                        [&](int p, int, int, C r) { F[p] = csub(cadd(r, r), B[p]); });
+                                        [&](int p, int, int, C r) { F[p] = cmk(fmaf_any(R(2), r.x, -B[p].x), fmaf_any(R(2), r.y, -B[p].y)); });
     sync();
   }
 }
@@ -208,12 +217,17 @@ __device__ __forceinline__ void basis_body(const LevelK<R> &L, const Gm2dWork<R>
                               [&](int p, int x, int y, C xl) {
     C v[M + 1];   // (zero outside the domain)
     v[0] = B[p];
-    if (M == 1) v[1] = cfma(sg, v[0], xl);
-    if (M >= 2) v[1] = cfma(sg, v[0], A[p]);
-    if (M == 2) v[2] = cfma(sg, A[p], xl);
+    auto shifted = [&](C q, C xq) {   // X q + s sigma q
+      C r = cmk(fmaf_any(sg.x, q.x, xq.x), fmaf_any(sg.x, q.y, xq.y));
+      if (sg.y != R(0)) r = cmk(fmaf_any(-sg.y, q.y, r.x), fmaf_any(sg.y, q.x, r.y));
+      return r;
+    };
+    if (M == 1) v[1] = shifted(v[0], xl);
+    if (M >= 2) v[1] = shifted(v[0], A[p]);
+    if (M == 2) v[2] = shifted(A[p], xl);
     if (M == 3) {
-      v[M - 1] = cfma(sg, A[p], cscale(cadd(F[p], v[0]), R(0.5)));
-      v[M] = cfma(sg, F[p], xl);
+      v[M - 1] = shifted(A[p], cscale(cadd(F[p], v[0]), R(0.5)));
+      v[M] = shifted(F[p], xl);
     }
     gram_point<R, M, PAIR>(acc, v);
     if (STORE && x < L.N && y < L.N) {
