@@ -18,6 +18,9 @@
 // sweep 633 -> 305; 85 to 90 % of each is the FP64 pipe (a warp's instruction takes
 // 64 cycles).  Runs of 32 rows, one warp each, took 161 / 327 / 258 / 348: blocks of
 // general strips (layers) cost twice the others' work and set a single wave's time.
+// A sequence of operator, adjoint operator, sweep, restriction, correction and coarse
+// sweep on one right-hand side takes 1397 us at 2047^2 (2297), 420 at 1023^2 (605),
+// 140 at 511^2 (181), 64 with four at 127^2 (78) and 70 with sixteen at 63^2 (78).
 #include "hh_kernels.cuh"
 
 #include <algorithm>
@@ -179,7 +182,8 @@ __global__ void __launch_bounds__(256) k_walk2d(Walk2dArgs<R> A) {
   const LevelK<R> &L = A.L;
   const int N = L.N, strips = (N + OW - 1) / OW, runs = (N + A.rows - 1) / A.rows;
   double acc = 0.0;
-  for (int i = blockIdx.x * 8 + warp; i < strips * runs; i += gridDim.x * 8) {
+  const int nw = blockDim.x >> 5;
+  for (int i = blockIdx.x * nw + warp; i < strips * runs; i += gridDim.x * nw) {
     const int run = i / strips, xa = (i - run * strips) * OW - F, x = xa + lane;
     const int y0 = run * A.rows, y1 = min(N, y0 + A.rows);
     const bool own = lane >= F && lane < F + OW && x < N;
@@ -193,15 +197,22 @@ __global__ void __launch_bounds__(256) k_walk2d(Walk2dArgs<R> A) {
   }
 }
 
-// Rows per run: at most 32; short enough for about 64 warps per SM, several blocks
-// each, which evens out the general strips' extra work (figures above).
+// Rows per run, at most 32: short enough for about 64 warps per SM, several blocks
+// each, which evens out the general strips' extra work (figures above); but up to 8
+// as long as 16 warps per SM are left, since a run's first rows are loaded, and the
+// restriction's residual is formed, twice.
 template <typename R, int KIND>
 void launch_walk2d(Walk2dArgs<R> a, int batch, int blocks, cudaStream_t s) {
   const int N = a.L.N, strips = (N + strip_cols<KIND>() - 1) / strip_cols<KIND>();
-  const long long r = (long long)N * strips * batch / (64 * 152);
+  const long long all = (long long)N * strips * batch, full = all / (64 * 152);
+  const long long r = std::max(full, std::min<long long>(8, all / (16 * 152)));
   a.rows = (int)std::min<long long>(32, std::max<long long>(2, r)) & ~1;
-  if (!blocks) blocks = (strips * ((N + a.rows - 1) / a.rows) + 7) / 8;
-  k_walk2d<R, KIND><<<dim3(blocks, batch), 256, 0, s>>>(a);
+  // two warps per block: with eight a few SMs got a block more than the others at
+  // small sizes (four at 127^2: the sequence 83 us instead of 64).  With partial
+  // sums the number of blocks is the caller's
+  const int threads = blocks ? 256 : 64;
+  if (!blocks) blocks = (strips * ((N + a.rows - 1) / a.rows) + 1) / 2;
+  k_walk2d<R, KIND><<<dim3(blocks, batch), threads, 0, s>>>(a);
 }
 
 template <typename R> void smooth2d(const LevelK<R> &L, const typename Cx<R>::T *u_in, int zero_mode,
