@@ -290,12 +290,11 @@ def run_ours(args):
                     "traffic": None, "bytes_per_point": bpp,
                     "launch_ms": {KERNELS3[k]: v for k, v in kt3.items()}}
     if args.smoother == "gmres":
-        # one level-0 GMRES(3) smoothing step (start, 3 Arnoldi steps, update),
-        # timed live back to back; a k^2 field adds 4 B per operator application
+        # one level-0 GMRES(3) smoothing step, timed live back to back
         ms = ct.c_double()
         B.check(B.lib().hh_time_kernel(mg._h, 6, 0, 1, 20, ct.byref(ms),
                                        ct.c_void_p(stream.cuda_stream)))
-        bpp = (GMRES_STEP_BYTES + (0.0 if kconst else 16.0)) * (1.0 if mixed else 2.0)
+        bpp = gmres_step_bytes(dim, kconst, mixed)
         achieved = bpp * pts / (ms.value * 1e-3) / 1e9
         roofline = {"bound": "hbm", "kernel": "gmres_step_level0", "achieved": achieved,
                     "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
@@ -454,14 +453,16 @@ def stored_traffic(workload, precision, kernel):
     return json.loads(tf.read_text()).get(f"{workload}:{precision}:{kernel}")
 
 
-# Algorithmic bytes per point of one GMRES(3) smoothing step on a level
-# (complex64 vectors, constant k; each kernel reads and writes its vectors
-# once): start: u, f -> q_0 (24 B); Arnoldi steps J = 0, 1: q_0..q_J -> w
-# (8 (J + 2)); orthogonalisations J = 0, 1: w, q_0..q_J -> q_{J+1}
-# (8 (J + 3)); the last Arnoldi step reads q_0..q_2 and forms only sums
-# (24 B; |q_3| follows from them); update: u, q_0..q_2 -> u (40 B).
-# Sum: 184 B.
-GMRES_STEP_BYTES = 184.0
+def gmres_step_bytes(dim, kconst, mixed):
+    """Algorithmic bytes per point of one GMRES(3) smoothing step on a level, each
+    kernel reading and writing its vectors once.  2-D complex64: two kernels that read
+    u, f (the basis is formed in both), u written: 40 B; complex128 stores the basis
+    instead: u, f in, q_0..q_2 out, u, q_0..q_2 in, u out: 160 B.  3-D: q_0, q_1 and q_2
+    by a kernel each, the Gram sums, the update: 128 or 256 B.  A k^2 field is read
+    once per kernel that forms products."""
+    if dim == 2:
+        return (40.0 if mixed else 160.0) + (0.0 if kconst else 8.0)
+    return (128.0 + (0.0 if kconst else 16.0)) * (1.0 if mixed else 2.0)
 
 
 def gmres_record(w, args, k2_t, f, stream, flush):
@@ -485,7 +486,7 @@ def gmres_record(w, args, k2_t, f, stream, flush):
     B.check(B.lib().hh_time_kernel(mg._h, 6, 0, 1, 20, ct.byref(ms), sp))
     step_ms = ms.value
     peak, peak_kind = measured_peaks()
-    bpp = GMRES_STEP_BYTES * (1.0 if mixed else 2.0)
+    bpp = gmres_step_bytes(dim, not torch.is_tensor(k2_t), mixed)
     achieved = bpp * pts / (step_ms * 1e-3) / 1e9
     flush.fill_(1.0)
     e0 = torch.cuda.Event(enable_timing=True)
