@@ -340,11 +340,11 @@ hh_status hh_coarse_solve(hh_handle *h, const void *f_dev, void *e_dev,
  *   kernel 1: residual + full-weighting restriction on `level`
  *   kernel 2: correction + post-smoothing sweep on `level`
  *   kernel 3: FP64 refinement residual on level 0 (MIXED handles only)
- *   kernel 4: the single-block kernel of the small levels (fused 2-D path,
- *             or the one-block tail of GMRES smoothing)
+ *   kernel 4: the small levels (fused 2-D path: the dense tail operator or the
+ *             single-block kernel; the one-block tail of GMRES smoothing)
  *   kernel 5: one whole V-cycle (no stop test), replayed as a CUDA graph
  *   kernel 6: one GMRES(m) smoothing step on `level` from a nonzero iterate
- *             (its start, m Arnoldi steps and update; GMRES handles only)
+ *             (basis, Gram matrix and update; GMRES handles only)
  * Kernels 0-2, 4-6 run in the handle's precision.  Workspace contents are
  * overwritten (the handle stays valid).  For benchmarks and profiles. */
 hh_status hh_time_kernel(hh_handle *h, int kernel, int level, int batch,

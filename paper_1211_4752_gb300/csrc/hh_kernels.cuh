@@ -1,9 +1,9 @@
 // Point-wise stencil kernels of the level-dependent Helmholtz multigrid,
 // templated on the real type R (float: complex64 cycles, double:
 // complex128) and the dimension DIM (2: 5-point, 3: 7-point).  They serve
-// the 3-D cycle, cycles with more than one sweep, the step-by-step entry
-// points and the FP64 refinement residual; the fused 2-D cycle kernels live
-// in hh_fused2d.cuh.  Included by hh_kernels_2d.cu / hh_kernels_3d.cu.
+// the 3-D cycles and step-by-step entry points and the FP64 refinement residual;
+// the 2-D steps are walking warps (hh_kernels_2d.cu), the fused 2-D cycle kernels
+// live in hh_fused2d.cuh.  Included by hh_kernels_2d.cu / hh_kernels_3d.cu.
 //
 // Layout (see LevelK): right-hand side b of a batch at offset b * S, rows of
 // pitch P; blockIdx.y selects b; threads walk the interior points.
