@@ -191,7 +191,9 @@ k_fg_restart(KrylovWork k, int au_zero, int first, int trust_est, SolveState *st
   const size_t off = (size_t)b * k.S;
   const double2 *f = k.F + off, *au = k.au + off;
   void *r = static_cast<typename KT<R>::C *>(k.V) + off;
-  R r2 = 0, f2 = 0;   // norms of the values rounded to R
+  // norms of the values rounded to R, in FP64: a restart's residual is tol |f|, whose
+  // FP32 squares vanish for sources of 1e-15 and less
+  double r2 = 0.0, f2 = 0.0;
   for_range<2 * kEpt>(block_range<R>(k), [&](long long u) {
     Unit<R> o;
 #pragma unroll
@@ -199,14 +201,14 @@ k_fg_restart(KrylovWork k, int au_zero, int first, int trust_est, SolveState *st
       const double2 fv = f[u * kPer + t];
       const double2 v = au_zero ? fv : csub(fv, au[u * kPer + t]);
       o.c[t] = KT<R>::make(v);
-      r2 += cabs2(o.c[t]);
-      if (first) f2 += cabs2(au_zero ? o.c[t] : KT<R>::make(fv));
+      r2 += cabs2(to_d(o.c[t]));
+      if (first) f2 += cabs2(to_d(au_zero ? o.c[t] : KT<R>::make(fv)));
     }
     stu<R>(r, u, o);
   });
   __shared__ BlockSums bs;
-  warp_deposit(bs, 0, r2, (R)0);
-  warp_deposit(bs, 1, f2, (R)0);
+  warp_deposit(bs, 0, r2, 0.0);
+  warp_deposit(bs, 1, f2, 0.0);
   flush_block_sums(bs, k.parts, b, 2);
   if (!arrive_last(k.counter, b)) return;
   const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
