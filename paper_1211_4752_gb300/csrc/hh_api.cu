@@ -144,8 +144,11 @@ struct hh_handle {
   int sms = 0;                      // SMs of the device
   void *gm2_parts = nullptr;        // GMRES smoothing: partial Gram matrices of a step,
   int *gm2_zero = nullptr;          // whether it started from zero (per right-hand side),
+  float *gm2_mag = nullptr;         // complex64: magnitude of the level-0 residual and the
+  float *gm2_g = nullptr;           // scale of the step's sums (hh_cheb.cuh),
   double *gm2_coef = nullptr;       // complex128: coefficients and their correction's sums
   double *gm2_parts2 = nullptr;
+  double anorm = 0.0;               // bound of the level-0 operator's norm (GMRES smoothing)
   int pw3d = 0;                     // 3-D: point-wise kernels instead of the tile-staged ones
   cudaStream_t side = nullptr;      // branch of the stop test in the fused cycle
   cudaStream_t grp = nullptr;       // this handle's stream in a group solve (lazy)
@@ -362,6 +365,9 @@ template <typename R> Gm2dLevel<R> gm2d_level(hh_handle *h, int l, int dir) {
   g.s = (R)v.gs;
   g.w.parts = reinterpret_cast<typename GramSum<R>::T *>(h->gm2_parts);
   g.w.zflag = h->gm2_zero;
+  g.w.mag = h->gm2_mag;
+  g.w.g = h->gm2_g;
+  g.w.track = l == 0;
   g.w.q = work<R>(h).gq[l];
   g.w.qs = (size_t)v.S * h->max_batch;
   g.w.coef = h->gm2_coef;
@@ -1028,7 +1034,7 @@ hh_status solve_core(hh_handle *h, int dir, const double2 *rhs,
     HH_TRY(copy_to_pitched(h, 0, h->u64[0], guess, batch, sizeof(double2), cudaMemcpyDeviceToDevice, s));
   refine_dispatch(h, dir, h->u64[0], guess ? 0 : 1, nullptr, h->u64[1], batch, s);
   cur = 1;
-  launch_check_outer(h->st, h->partials, h->params, h->flag, s);
+  launch_check_outer(h->st, h->partials, h->params, h->flag, h->gm2_mag, s);
   h->fixed_kernels += 2;
   for (int it = 0; it < h->opt.max_cycles + 2; ++it) {
     HH_CK(cudaMemcpyAsync(h->flag_h, h->flag, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1038,7 +1044,7 @@ hh_status solve_core(hh_handle *h, int dir, const double2 *rhs,
     HH_TRY(run_loop(h, HH_MIXED, dir, batch, s));
     refine_dispatch(h, dir, h->u64[cur], 0, h->w32.u_post[0], h->u64[1 - cur], batch, s);
     cur = 1 - cur;
-    launch_check_outer(h->st, h->partials, h->params, h->flag, s);
+    launch_check_outer(h->st, h->partials, h->params, h->flag, h->gm2_mag, s);
     h->fixed_kernels += 2;
   }
   launch_finish(h->st, h->u64[cur], l0, out, d0, h->dim, batch, s);
@@ -1800,6 +1806,7 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
     a.u = work<R>(h).u_post[t0];
     a.lay = lay_of(h, t0);
     a.inv = h->inv[dir];
+    a.mag = h->gm2_mag;
     a.mm = h->m;
     if constexpr (std::is_same<R, float>::value) h->gta32[dir] = a;
     else h->gta64[dir] = a;
@@ -1986,6 +1993,11 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     h->gm2_parts = q;
     HH_TRY(dev_alloc_n(h, &h->gm2_zero, (size_t)B));
     HH_CK(cudaMemsetAsync(h->gm2_zero, 0, (size_t)B * sizeof(int), s));
+    if (h->opt.precision == HH_MIXED) {
+      HH_TRY(dev_alloc_n(h, &h->gm2_mag, (size_t)B));
+      HH_TRY(dev_alloc_n(h, &h->gm2_g, (size_t)B));
+      HH_CK(cudaMemsetAsync(h->gm2_mag, 0, (size_t)B * sizeof(float), s));
+    }
     if (h->opt.precision == HH_FP64) {
       HH_TRY(dev_alloc_n(h, &h->gm2_coef, (size_t)kGm2dCoef * B));
       HH_TRY(dev_alloc_n(h, &h->gm2_parts2, (size_t)kGm2dCorr * 8 * B));
@@ -2076,6 +2088,9 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     // spectrum of a level: 2 dim c_0 - beta k^2 plus the neighbours' part,
     // |2 dim c_0| at most (coarse k^2 is injected from the fine field)
     const double kmid = 0.5 * (krange[0] + krange[1]), krad = 0.5 * (krange[1] - krange[0]);
+    const double c00 = std::hypot(h->lv[0].c0_64[0].x, h->lv[0].c0_64[0].y);
+    h->anorm = 4.0 * dim * c00 + std::hypot(h->lv[0].beta64[0].x, h->lv[0].beta64[0].y) *
+                                     std::max(std::fabs(krange[0]), std::fabs(krange[1]));
     for (LevelHost &v : h->lv) {
       for (int d = 0; d < 2; ++d) {
         v.sig64[d].x = 2.0 * dim * v.c0_64[d].x - v.beta64[d].x * kmid;
@@ -2308,7 +2323,7 @@ hh_status group_solve_impl(hh_group *g, const hh_group_item *items, double tol, 
       HH_TRY(copy_to_pitched(h, 0, h->u64[0], items[p].u_dev, B, sizeof(double2),
                              cudaMemcpyDeviceToDevice, s));
     refine_dispatch(h, 0, h->u64[0], guess ? 0 : 1, nullptr, h->u64[1], B, s);
-    launch_check_outer(h->st, h->partials, h->params, h->flag, s);
+    launch_check_outer(h->st, h->partials, h->params, h->flag, h->gm2_mag, s);
     cur[p] = 1;
   }
   HH_CK(cudaMemsetAsync(g->copies, 0, sizeof(unsigned int), s));
@@ -2337,7 +2352,7 @@ hh_status group_solve_impl(hh_group *g, const hh_group_item *items, double tol, 
       hh_handle *h = g->h[p];
       refine_dispatch(h, 0, h->u64[cur[p]], 0, h->w32.u_post[0], h->u64[1 - cur[p]], g->batch[p], s);
       cur[p] = 1 - cur[p];
-      launch_check_outer(h->st, h->partials, h->params, h->flag, s);
+      launch_check_outer(h->st, h->partials, h->params, h->flag, h->gm2_mag, s);
       fixed += 2;
     }
   }
@@ -2531,6 +2546,8 @@ hh_status fgmres_core(hh_handle *h, const double2 *rhs, double2 *u, int guess, i
   P.batch = batch;
   P.nparts = k.nblk;
   HH_CK(cudaMemcpyAsync(h->params, h->params_h, sizeof(SolveParams), cudaMemcpyHostToDevice, s));
+  // (the preconditioner's right-hand sides have norm one)
+  if (h->gm2_mag) HH_CK(cudaMemsetAsync(h->gm2_mag, 0, (size_t)batch * sizeof(float), s));
   HH_CK(cudaMemsetAsync(h->err, 0, sizeof(int), s));
   HH_CK(cudaMemsetAsync(h->copies, 0, sizeof(unsigned int), s));
   cudaGraphExec_t ex;
@@ -3056,8 +3073,12 @@ hh_status hh_cycles(hh_handle *h, const void *rhs_dev, void *u_dev, int batch,
     HH_TRY(copy_to_dense(h, 0, u_dev, h->w64.u_post[0], batch, sizeof(double2), cudaMemcpyDeviceToDevice, s));
   } else {
     const Lay l0 = lay_of(h, 0), d0 = lay_dense(h, 0);
-    launch_c128_to_c64((const double2 *)rhs_dev, d0, h->w32.f[0], l0, h->dim, batch, s);
-    launch_c128_to_c64((const double2 *)u_dev, d0, h->w32.u_post[0], l0, h->dim, batch, s);
+    // GMRES smoothing: |f - A u| is at most |f| + ||A|| |u|, component by component
+    float *mag = h->gm2_mag;
+    if (mag) HH_CK(cudaMemsetAsync(mag, 0, (size_t)batch * sizeof(float), s));
+    launch_c128_to_c64((const double2 *)rhs_dev, d0, h->w32.f[0], l0, h->dim, batch, mag, 1.f, s);
+    launch_c128_to_c64((const double2 *)u_dev, d0, h->w32.u_post[0], l0, h->dim, batch, mag,
+                       (float)h->anorm, s);
     for (int k = 0; k < ncycles; ++k)
       cycle_dispatch<float>(h, 0, batch, ZERO_NONE, CHECK_NONE, 0, s);
     launch_c64_to_c128(h->w32.u_post[0], l0, (double2 *)u_dev, d0, h->dim, batch, s);

@@ -11,6 +11,10 @@
 //     N y = b,   N_ij = <a_i, a_j>,  b_i = <a_i, r>,
 // whose entries, with |r|^2, are the Gram matrix of (r, a_0 .. a_{m-1}).  Then
 //     z = s sum y_j q_j.
+// complex64: the sums are those of g r and its basis, g a power of two that keeps the
+// level-0 residual's norm within 2^-24 .. 2^25 (gram_scale): the products are squares,
+// which leave FP32's range at 1e-19 and 1e19 (the pairs' second values at 1e-12).  y
+// does not depend on g.
 // (The new residual r - sum y_j a_j is not taken from the basis: in complex64 it
 // would miss the rounding of u + z, which f - A (u + z) contains and the coarse
 // levels correct; the cycles' error against FP64 was 2 to 4 times larger.)
@@ -90,6 +94,31 @@ template <bool P> __device__ __forceinline__ void gram_add(GramAcc<float, P> &a,
 __device__ __forceinline__ void gram_add(GramAcc<double, false> &a, double v) { a.h += v; }
 __device__ __forceinline__ double gram_value(float2 v) { return (double)v.x + (double)v.y; }   // for the stop test
 __device__ __forceinline__ double gram_value(double v) { return v; }
+
+// g of a right-hand side from the estimate m[b] of its level-0 residual's magnitude:
+// 1 for an m of 2^-24 .. 2^25 and where there is none (0, infinity, NaN), else the power
+// of two that brings m to [1, 2).
+__device__ __forceinline__ float gram_scale(const float *m, int b) {
+  const float v = m[b];
+  if (!(v > 0.f) || !(v < 3e38f)) return 1.f;
+  const int e = min(80, max(-80, ((__float_as_int(v) >> 23) & 255) - 127));
+  return e >= -24 && e <= 24 ? 1.f : __int_as_float((127 - e) << 23);
+}
+template <typename R> __device__ __forceinline__ R gram_scale_of(const float *m, int b) {
+  if constexpr (sizeof(R) == 4) return gram_scale(m, b);
+  else return R(1);
+}
+__device__ __forceinline__ float gram_rcp(float g) { return __int_as_float((254 << 23) - __float_as_int(g)); }   // 1 / g
+// |r|^2 from the sum of |g r|^2
+template <typename S> __device__ __forceinline__ double gram_unscaled(S sum, float g) {
+  const double i = (double)gram_rcp(g);
+  return gram_value(sum) * i * i;
+}
+// The next step's estimate from the sum of |g q_0|^2 of this one (left where that
+// says nothing)
+__device__ __forceinline__ void gram_estimate(float *m, int b, float2 sum, float g) {
+  if (sum.x > 0.f && sum.x < 3e38f) m[b] = sqrtf(sum.x) * gram_rcp(g);
+}
 
 // Real numbers of the Gram matrix of m + 1 vectors, and that count rounded up
 // to a power of two: entry i <= m is |v_i|^2; pair (i < j), counted in the order

@@ -53,9 +53,10 @@ template <int DIM, typename F> __device__ __forceinline__ void tail_points(int N
 }
 
 // One GMRES(M) step on level K (iterate U, right-hand side F; zero: U is taken
-// as zero).  res: Q0 holds f - A u of the new iterate afterwards.
+// as zero; g: scale of the vectors, hh_cheb.cuh).  res: Q0 holds f - A u of the new
+// iterate afterwards.
 template <typename R, int DIM, int M>
-__device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s,
+__device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s, R g,
                              typename Cx<R>::T *U, const typename Cx<R>::T *F,
                              typename Cx<R>::T *Q0, typename Cx<R>::T *Q1, typename Cx<R>::T *Q2,
                              bool zero, bool res,
@@ -80,7 +81,7 @@ __device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s,
         stencil<R, DIM>(K, x, y, z, get, Au, D, uc);
         r = csub(r, Au);
       }
-      Q0[p] = r;
+      Q0[p] = cscale(r, g);
     });
   }
   __syncthreads();
@@ -129,7 +130,7 @@ __device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s,
     __syncwarp();
     if (lane < NQP) sums[lane] = gram_store(v);
     __syncwarp();
-    gram_solve<R, M>(sums, s, gram_tol<R>(PAIR), sc);
+    gram_solve<R, M>(sums, sizeof(R) == 4 ? s * (R)gram_rcp((float)g) : s, gram_tol<R>(PAIR), sc);
   }
   __syncthreads();
   if constexpr (sizeof(R) == 8) {
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
   for (int j = threadIdx.x; j < mm * mm; j += TB) sinv[j] = A.inv[j];
   griddep_wait();
   griddep_launch_dependents();
+  const R g = gram_scale_of<R>(A.mag, b);   // (in flight early)
   if (!__syncthreads_and(!(st && !st[b].active))) return;   // one decision per block
   {
     const int N = A.lv[0].K.N;
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
     C *U = cm + A.lv[i].offU;
     const C *F = cm + A.lv[i].offF;
     for (int s = 0; s < A.nu1; ++s)
-      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, U, F, Q0, Q1, Q2, s == 0,
+      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, g, U, F, Q0, Q1, Q2, s == 0,
                               s == A.nu1 - 1, sums, &sc);
     {
       const C *r = Q0;
@@ -304,7 +306,7 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
     });
     __syncthreads();
     for (int s = 0; s < A.nu2; ++s)
-      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, U, F, Q0, Q1, Q2, false, false,
+      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, g, U, F, Q0, Q1, Q2, false, false,
                               sums, &sc);
   }
   {

@@ -32,6 +32,7 @@ template <typename R> struct GmTailArgs {
   typename Cx<R>::T *u;        // its correction
   Lay lay;
   const double2 *inv;          // inverse of the coarsest operator (FP64, mm x mm)
+  const float *mag;            // complex64: Gm2dWork::mag
   int mm;
 };
 template <typename R, int DIM> size_t gmres_tail_smem(const int *N, int nl, int m);

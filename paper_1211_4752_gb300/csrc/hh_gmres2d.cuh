@@ -182,19 +182,19 @@ template <int M, int T> struct BasisTile {
   static constexpr int NT = round32(imax(E * E, 2 * T * T));
 };
 
-// q_0 .. q_{M-1} of a tile's points in shared memory: q_j is valid j points
-// inside the E x E region.  sw: the iterate on (E + 2)^2.  bar: barrier id of
+// q_0 .. q_{M-1} (times g) of a tile's points in shared memory: q_j is valid j
+// points inside the E x E region.  sw: the iterate on (E + 2)^2.  bar: barrier id of
 // the `nt` threads that take part.
 template <typename R, int M, int E>
 __device__ __forceinline__ void tile_basis(const PointOp<R> &op, typename Cx<R>::T fv,
                                            const typename Cx<R>::T *sw,
                                            typename Cx<R>::T (*sq)[E * E],
-                                           typename Cx<R>::T sigma, R s, int tx, int ty, bool mine,
+                                           typename Cx<R>::T sigma, R s, R g, int tx, int ty, bool mine,
                                            int bar, int nt) {
   using C = typename Cx<R>::T;
   constexpr int W = E + 2;
   const int o = ty * E + tx;
-  if (mine) sq[0][o] = op.resid(fv, sw + (ty + 1) * W + tx + 1, W);
+  if (mine) sq[0][o] = cscale(op.resid(fv, sw + (ty + 1) * W + tx + 1, W), g);
 #pragma unroll
   for (int j = 1; j < M; ++j) {
     bar_sync(bar, nt);
@@ -230,15 +230,19 @@ k_gm2d_basis_tile(LevelK<R> L, typename Cx<R>::T sigma, R s, Gm2dIn<R> in, Gm2dW
   gp.load(L, half < 2 ? x0 + ix : -1, y0 + iy);
   griddep_wait();
   griddep_launch_dependents();
+  const R g = gram_scale_of<R>(wk.mag, b);   // (in flight early)
   if (!__syncthreads_and(!(st && !st[b].active))) return;   // one decision per block
   const bool zero = __syncthreads_or(in.zero_mode == ZERO_ALL ||
                                      (in.zero_mode == ZERO_FLAG && st && st[b].zero)) != 0;
-  if (blockIdx.x == 0 && tid == 0) wk.zflag[b] = zero;
+  if (blockIdx.x == 0 && tid == 0) {
+    wk.zflag[b] = zero;
+    if (sizeof(R) == 4) wk.g[b] = (float)g;
+  }
   const C fv = op.in ? in.f[(size_t)b * L.S + (size_t)(y0 - M + ty) * L.P + x0 - M + tx] : czero<C>();
   for (int i = tid; i < W * W; i += NT)
     sw[i] = start_at<R, CORR>(L, in, b, zero, x0 - M - 1 + i % W, y0 - M - 1 + i / W);
   __syncthreads();
-  tile_basis<R, M, E>(op, fv, sw, sq, sigma, s, tx, ty, mine, 0, NT);
+  tile_basis<R, M, E>(op, fv, sw, sq, sigma, s, g, tx, ty, mine, 0, NT);
   A acc[NQP];
 #pragma unroll
   for (int i = 0; i < NQP; ++i) acc[i].zero();
@@ -274,9 +278,9 @@ k_gm2d_basis_tile(LevelK<R> L, typename Cx<R>::T sigma, R s, Gm2dIn<R> in, Gm2dW
     A t;
     t.zero();
     for (int i = 0; i < HW; ++i) gram_add(t, sums[(w0 + i) * H + tid % H]);
-    const S g = gram_store(t);
-    wk.parts[((size_t)b * gridDim.x + blockIdx.x) * NQP + tid] = g;
-    if (check && tid == 0) check[(size_t)b * gridDim.x + blockIdx.x] = gram_value(g);
+    const S q = gram_store(t);
+    wk.parts[((size_t)b * gridDim.x + blockIdx.x) * NQP + tid] = q;
+    if (check && tid == 0) check[(size_t)b * gridDim.x + blockIdx.x] = gram_unscaled(q, (float)g);
   }
 }
 
@@ -318,10 +322,13 @@ k_gm2d_update_tile(LevelK<R> L, typename Cx<R>::T sigma, R s, Gm2dIn<R> in, Gm2d
   __syncthreads();
   // the last warp solves for the coefficients while the others form the basis
   if (tid >= NC) {
-    if constexpr (sizeof(R) == 4) solve_warp<R, M>(sums, NT / 32, s, tol, &sc);
+    if constexpr (sizeof(R) == 4) {
+      solve_warp<R, M>(sums, NT / 32, s, tol, &sc);
+      if (wk.track && blockIdx.x == 0 && tid == NC) gram_estimate(wk.mag, b, sums[0], wk.g[b]);
+    }
     else read_coef<M>(wk, b, nparts, s, tol, sums, &sc);
   }
-  else tile_basis<R, M, E>(op, fv, sw, sq, sigma, s, tx, ty, mine, 1, NC);
+  else tile_basis<R, M, E>(op, fv, sw, sq, sigma, s, R(1), tx, ty, mine, 1, NC);
   __syncthreads();
   const int o = ty * E + tx, ow = (ty + 1) * W + tx + 1;
   const bool have = mine && tx >= M - 1 && tx < E - (M - 1) && ty >= M - 1 && ty < E - (M - 1);

@@ -25,10 +25,14 @@ template <typename R> struct Gm2dIn {
 };
 
 // Workspace: partial Gram matrices [b][block][NQP], whether the basis kernel
-// took the iterate as zero ([b]), and (complex128) the stored basis.
+// took the iterate as zero ([b]), complex64: the scale of its sums ([b]), and
+// (complex128) the stored basis.
 template <typename R> struct Gm2dWork {
   typename GramSum<R>::T *parts;
   int *zflag;
+  float *mag;                   // complex64: estimate of the level-0 residual's magnitude
+  float *g;                     // and the scale that the step's basis kernel took from it
+  int track;                    // the step is on level 0: its |r| is the next estimate
   typename Cx<R>::T *q;         // complex128: q_0 .. q_{m-1} and X q_{m-1}, stride qs,
   size_t qs;
   double *coef;                 // the solved coefficients ([b][kGm2dCoef]) and the

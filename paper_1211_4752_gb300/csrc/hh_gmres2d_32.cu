@@ -60,7 +60,7 @@ template <typename R, int M, int NX, int MODE, bool CORR, bool FROWS = false> st
   const LevelK<R> &L;
   const Gm2dIn<R> &in;
   C sigma;
-  R s;
+  R s, g;                  // g: factor of q_0
   int x, wmax, fmax;
   bool zero, inx;          // inx: the lane's column is inside the domain
   const C *u, *f, *e;
@@ -80,8 +80,8 @@ template <typename R, int M, int NX, int MODE, bool CORR, bool FROWS = false> st
   C exB;
 
   __device__ __forceinline__ March(const LevelK<R> &L_, const Gm2dIn<R> &in_, C sigma_, R s_,
-                                   int b, bool zero_, int x_)
-      : L(L_), in(in_), sigma(sigma_), s(s_), x(x_), zero(zero_) {
+                                   R g_, int b, bool zero_, int x_)
+      : L(L_), in(in_), sigma(sigma_), s(s_), g(g_), x(x_), zero(zero_) {
     N = L.N;
     P = L.P;
     inx = MODE != GENERAL || (unsigned)x < (unsigned)N;
@@ -220,7 +220,7 @@ template <typename R, int M, int NX, int MODE, bool CORR, bool FROWS = false> st
       pk[O] = load_k(y + 2);
     }
     if (FROWS) fr[S] = fv;
-    q0[S] = zero ? fv : resid(fv, w[S3], w[S], w[S1], y, k[S]);
+    q0[S] = cscale(zero ? fv : resid(fv, w[S3], w[S], w[S1], y, k[S]), g);
     w0(S, w[S]);
     hook(I0(), S, q0[S]);
     C xl = czero<C>();
@@ -347,11 +347,11 @@ constexpr int kMaxWarps = 16;   // per block: 128 registers per thread
 
 template <typename R, int M, bool PAIR, int MODE, bool CORR>
 __device__ __forceinline__ void basis_run(const LevelK<R> &L, const Gm2dIn<R> &in,
-                                          typename Cx<R>::T sigma, R s, int b, bool zero, int x,
+                                          typename Cx<R>::T sigma, R s, R g, int b, bool zero, int x,
                                           int y0, int y1, bool own,
                                           GramAcc<R, PAIR> (&acc)[Gram<M>::NQP]) {
   using C = typename Cx<R>::T;
-  March<R, M, M, MODE, CORR> m(L, in, sigma, s, b, zero, x);
+  March<R, M, M, MODE, CORR> m(L, in, sigma, s, g, b, zero, x);
   const C t = cscale(sigma, s);
   auto none0 = [](int, C) {};
   auto none = [](auto, int, C) {};
@@ -383,10 +383,14 @@ k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in
   const MarchWork work(L, rows, G::F, G::OW, M);
   griddep_wait();
   griddep_launch_dependents();
+  const R g = gram_scale_of<R>(wk.mag, b);   // (in flight early)
   if (!__syncthreads_and(!(st && !st[b].active))) return;   // one decision per block
   const bool zero = __syncthreads_or(in.zero_mode == ZERO_ALL ||
                                      (in.zero_mode == ZERO_FLAG && st && st[b].zero)) != 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) wk.zflag[b] = zero;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    wk.zflag[b] = zero;
+    wk.g[b] = g;
+  }
   GramAcc<R, PAIR> acc[NQP];
 #pragma unroll
   for (int i = 0; i < NQP; ++i) acc[i].zero();
@@ -396,9 +400,9 @@ k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in
     const bool uni = work.item(wi, L.N, strip, y0, y1);
     const int x = strip * G::OW - G::F + lane;
     if (y0 >= y1) continue;
-    if (!uni) basis_run<R, M, PAIR, GENERAL, CORR>(L, in, sigma, s, b, zero, x, y0, y1, own, acc);
-    else if (kconst) basis_run<R, M, PAIR, UNIFORM_K, CORR>(L, in, sigma, s, b, zero, x, y0, y1, own, acc);
-    else basis_run<R, M, PAIR, UNIFORM, CORR>(L, in, sigma, s, b, zero, x, y0, y1, own, acc);
+    if (!uni) basis_run<R, M, PAIR, GENERAL, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
+    else if (kconst) basis_run<R, M, PAIR, UNIFORM_K, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
+    else basis_run<R, M, PAIR, UNIFORM, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
   }
   // block sums, in a fixed order
   constexpr int SH = NQP == 16 ? 1 : 3;   // lane l holds quantity l >> SH
@@ -409,9 +413,9 @@ k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in
     GramAcc<R, PAIR> t;
     t.zero();
     for (int i = 0; i < nw; ++i) gram_add(t, sums[i * NQP + threadIdx.x]);
-    const S g = gram_store(t);
-    wk.parts[((size_t)b * gridDim.x + blockIdx.x) * NQP + threadIdx.x] = g;
-    if (check && threadIdx.x == 0) check[(size_t)b * gridDim.x + blockIdx.x] = gram_value(g);
+    const S q = gram_store(t);
+    wk.parts[((size_t)b * gridDim.x + blockIdx.x) * NQP + threadIdx.x] = q;
+    if (check && threadIdx.x == 0) check[(size_t)b * gridDim.x + blockIdx.x] = gram_unscaled(q, g);
   }
 }
 
@@ -445,7 +449,7 @@ __device__ __forceinline__ void update_run(const LevelK<R> &L, const Gm2dIn<R> &
                                            typename Cx<R>::T csc, const Lay &lc) {
   using C = typename Cx<R>::T;
   constexpr int NX = M - 1;
-  March<R, M, NX, MODE, CORR, REST> m(L, in, sigma, s, b, zero, x);
+  March<R, M, NX, MODE, CORR, REST> m(L, in, sigma, s, R(1), b, zero, x);
   const int N = L.N;
   const bool cown = REST && own && (x & 1) && (x - 1) / 2 < lc.N;
   C o[4], un[4];
@@ -492,6 +496,7 @@ k_gm2d_update(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> i
   if (!__syncthreads_and(!(st && !st[b].active))) return;
   const bool zero = wk.zflag[b] != 0;
   step_coef<R, M>(wk.parts + (size_t)b * nparts * NQP, nparts, s, tol, sums, &sc);
+  if (wk.track && blockIdx.x == 0 && threadIdx.x == 0) gram_estimate(wk.mag, b, sums[0], wk.g[b]);
   const C csc = cscale(cs, R(1.0 / 16.0));
   u_out += (size_t)b * L.S;
   if (REST) fc += (size_t)b * lc.S;

@@ -106,7 +106,7 @@ __device__ __forceinline__ void walk_z(const LevelK<R> &L, const Walk3<R> &W, co
   }
 }
 
-// Block sums of the Gram quantities into parts (and |q_0|^2 into check).
+// Block sums of the Gram quantities into parts (and |q_0|^2, unscaled, into check).
 template <typename R, int M, bool PAIR>
 __device__ __forceinline__ void store_gram(GramAcc<R, PAIR> (&acc)[Gram<M>::NQP],
                                            const Gm2dWork<R> &wk, int b, double *check) {
@@ -121,9 +121,10 @@ __device__ __forceinline__ void store_gram(GramAcc<R, PAIR> (&acc)[Gram<M>::NQP]
     GramAcc<R, PAIR> t;
     t.zero();
     for (int i = 0; i < NW; ++i) gram_add(t, sums[i * NQP + threadIdx.x]);
-    const S g = gram_store(t);
-    wk.parts[((size_t)b * gridDim.x + blockIdx.x) * NQP + threadIdx.x] = g;
-    if (check && threadIdx.x == 0) check[(size_t)b * gridDim.x + blockIdx.x] = gram_value(g);
+    const S q = gram_store(t);
+    wk.parts[((size_t)b * gridDim.x + blockIdx.x) * NQP + threadIdx.x] = q;
+    if (check && threadIdx.x == 0)
+      check[(size_t)b * gridDim.x + blockIdx.x] = gram_unscaled(q, sizeof(R) == 4 ? wk.g[b] : 1.f);
   }
 }
 
@@ -169,7 +170,8 @@ k_gm3d_correct(LevelK<R> L, const typename Cx<R>::T *u, const typename Cx<R>::T 
   }
 }
 
-// J = 0: q_0 = f - A w; J = 1: q_1 = X q_0; J = 2: q_2 = 2 X q_1 - q_0.
+// J = 0: q_0 = g (f - A w) (g: hh_cheb.cuh; 1 in complex128); J = 1: q_1 = X q_0;
+// J = 2: q_2 = 2 X q_1 - q_0.
 template <typename R, int J>
 __global__ void __launch_bounds__(kT3)
 k_gm3d_vector(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in, Gm2dWork<R> wk,
@@ -180,12 +182,16 @@ k_gm3d_vector(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> i
   const Column3<R> K(L, kconst, W);
   griddep_wait();
   griddep_launch_dependents();
+  const R g = J == 0 ? gram_scale_of<R>(wk.mag, b) : R(1);   // (in flight early)
   if (!__syncthreads_and(!(st && !st[b].active))) return;   // one decision per block
   C *q = wk.q + (size_t)b * L.S;
   if constexpr (J == 0) {
     const bool zero = __syncthreads_or(in.zero_mode == ZERO_ALL ||
                                        (in.zero_mode == ZERO_FLAG && st && st[b].zero)) != 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) wk.zflag[b] = zero;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      wk.zflag[b] = zero;
+      if (sizeof(R) == 4) wk.g[b] = (float)g;
+    }
     const C *f = in.f + (size_t)b * L.S;
     if (zero) {
       if (W.in)
@@ -196,6 +202,9 @@ k_gm3d_vector(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> i
         q[o] = cadd(csub(f[o], cmul(D, v)), nb);
       });
     }
+    // (seldom: with the multiplication in the loop 127^3 took 42 us instead of 35)
+    if (g != R(1) && W.in)
+      for (int z = W.z0; z < W.z1; ++z) q[z * W.plane + W.off] = cscale(q[z * W.plane + W.off], g);
   } else {
     const C *a = q + (size_t)(J - 1) * wk.qs;
     C *out = q + (size_t)J * wk.qs;
@@ -253,8 +262,10 @@ k_gm3d_update(LevelK<R> L, R s, const typename Cx<R>::T *u_in, Gm2dWork<R> wk, i
   griddep_launch_dependents();
   if (!__syncthreads_and(!(st && !st[b].active))) return;
   const bool zero = wk.zflag[b] != 0;
-  if constexpr (sizeof(R) == 4) {
-    step_coef<R, M>(wk.parts + (size_t)b * nparts * NQP, nparts, s, tol, sums, &sc);
+  if constexpr (sizeof(R) == 4) {   // (the stored q_j are g times the basis)
+    const float g = wk.g[b];
+    step_coef<R, M>(wk.parts + (size_t)b * nparts * NQP, nparts, s * gram_rcp(g), tol, sums, &sc);
+    if (wk.track && blockIdx.x == 0 && threadIdx.x == 0) gram_estimate(wk.mag, b, sums[0], g);
   } else {
     if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, tol, sums, &sc);
     __syncthreads();

@@ -118,9 +118,11 @@ void launch_inject(const double *kf, const Lay &lf, double *kc, const Lay &lc,
 void launch_norm2(const double2 *x, size_t stride, int batch, double *partials,
                   int nparts, cudaStream_t s);
 void launch_to_float(const double *x, float *y, size_t n, cudaStream_t s);
-// layout-converting copies between caller (dense) and library (pitched) arrays
+// layout-converting copies between caller (dense) and library (pitched) arrays.  mag:
+// mag[b] becomes at least `factor` times the largest component of right-hand side b
+// (or null)
 void launch_c128_to_c64(const double2 *x, const Lay &lx, float2 *y, const Lay &ly, int dim,
-                        int batch, cudaStream_t s);
+                        int batch, float *mag, float factor, cudaStream_t s);
 void launch_c64_to_c128(const float2 *x, const Lay &lx, double2 *y, const Lay &ly, int dim,
                         int batch, cudaStream_t s);
 void launch_state_init(SolveState *st, const double *partials,
@@ -133,8 +135,9 @@ void launch_check_inner(SolveState *st, const double *partials,
                         const SolveParams *P, int *flag,
                         unsigned long long cond, unsigned int *copies, const int *err,
                         cudaStream_t s);
+// mag: the residual's norm of every right-hand side that goes on (or null)
 void launch_check_outer(SolveState *st, const double *partials,
-                        const SolveParams *P, int *flag, cudaStream_t s);
+                        const SolveParams *P, int *flag, float *mag, cudaStream_t s);
 void launch_finish(const SolveState *st, const double2 *src, const Lay &ls, double2 *dst,
                    const Lay &ld, int dim, int batch, cudaStream_t s);
 void launch_grad_k2(const double2 *u, const double2 *lam, size_t pts,

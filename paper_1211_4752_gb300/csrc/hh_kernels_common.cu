@@ -46,21 +46,37 @@ __global__ void k_to_float(const double *__restrict__ x, float *__restrict__ y,
 
 // Layout-converting copies: point (x, y[, z]) of right-hand side b from
 // layout lx to layout ly (dense caller arrays <-> pitched library arrays).
+// (a right-hand side has fewer than 2^32 points: a 64-bit division would bound the
+// copies, which also take the maximum for the GMRES smoothing)
 __device__ __forceinline__ size_t lay_at(const Lay &l, int dim, size_t p, int b) {
-  const int x = (int)(p % l.N);
-  const size_t r = p / l.N;   // row index: y, or z * N + y in 3-D
+  const unsigned r = (unsigned)p / (unsigned)l.N;   // row index: y, or z * N + y in 3-D
+  const unsigned x = (unsigned)p - r * (unsigned)l.N;
   (void)dim;
-  return (size_t)b * l.S + r * l.P + x;
+  return (size_t)b * l.S + (size_t)r * l.P + x;
 }
 
 __global__ void k_c128_to_c64(const double2 *__restrict__ x, Lay lx,
-                              float2 *__restrict__ y, Lay ly, int dim) {
+                              float2 *__restrict__ y, Lay ly, int dim, float *mag, float factor) {
   const int b = blockIdx.y;
+  float m = 0.f;
   const size_t pts = dim == 2 ? (size_t)lx.N * lx.N : (size_t)lx.N * lx.N * lx.N;
   for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < pts;
        p += (size_t)gridDim.x * blockDim.x) {
     const double2 v = x[lay_at(lx, dim, p, b)];
-    y[lay_at(ly, dim, p, b)] = make_float2((float)v.x, (float)v.y);
+    const float2 w = make_float2((float)v.x, (float)v.y);
+    y[lay_at(ly, dim, p, b)] = w;
+    m = fmaxf(m, fmaxf(fabsf(w.x), fabsf(w.y)));
+  }
+  if (!mag) return;
+  // (of nonnegative floats the bits order the values; few blocks raise the maximum)
+  const int most = __reduce_max_sync(0xffffffffu, __float_as_int(fminf(m * factor, 3e38f)));
+  __shared__ int ws[8];
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = most;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int v = __reduce_max_sync(0xffffffffu, threadIdx.x < (blockDim.x >> 5) ? ws[threadIdx.x] : 0);
+    int *p = reinterpret_cast<int *>(mag + b);
+    if (threadIdx.x == 0 && v > *(volatile int *)p) atomicMax(p, v);
   }
 }
 
@@ -92,7 +108,7 @@ __device__ void for_each_rhs(const SolveParams *P, const double *partials,
     if (!use) continue;
     const double r2 = warp_sum(partials + (size_t)b * P->nparts, P->nparts, lane);
     if (lane == 0) {
-      body(s, r2);
+      body(s, r2, b);
       st[b] = s;
       if (s.active) atomicOr(&any, 1);
     }
@@ -143,7 +159,7 @@ __global__ void k_check(SolveState *st, const double *partials, const SolveParam
                         unsigned long long cond, unsigned int *copies, const int *err) {
   __shared__ int any_s;
   const bool timeout = err && *(volatile const int *)err;
-  auto body = [&](SolveState &s, double r2) {
+  auto body = [&](SolveState &s, double r2, int) {
     if (timeout) {
       s.status = HH_ERR_TIMEOUT; s.active = 0; s.done = 1;
     } else if (MODE == CHECK_MODE_CYCLE) {
@@ -162,9 +178,9 @@ __global__ void k_check(SolveState *st, const double *partials, const SolveParam
 
 // Outer stop test of the FP64 refinement: r2 = ||f - A_0 u64||^2.
 __global__ void k_check_outer(SolveState *st, const double *partials,
-                              const SolveParams *P, int *flag) {
+                              const SolveParams *P, int *flag, float *mag) {
   __shared__ int any_s;
-  auto body = [&](SolveState &s, double r2) {
+  auto body = [&](SolveState &s, double r2, int b) {
     const double rho = sqrt(r2 / s.fnorm2);
     s.rnorm2 = r2;
     if (!(rho <= P->div_limit)) {
@@ -175,6 +191,7 @@ __global__ void k_check_outer(SolveState *st, const double *partials,
       s.status = HH_ERR_NOT_CONVERGED; s.active = 0; s.done = 1;
     } else {
       s.refinements += 1; s.active = 1; s.zero = 1; s.inner = 0;
+      if (mag) mag[b] = (float)fmin(sqrt(r2), 3e38);
     }
   };
   for_each_rhs(P, partials, st, false, body, &any_s);
@@ -244,9 +261,9 @@ void launch_to_float(const double *x, float *y, size_t n, cudaStream_t s) {
   k_to_float<<<grid_cap(n), 256, 0, s>>>(x, y, n);
 }
 void launch_c128_to_c64(const double2 *x, const Lay &lx, float2 *y, const Lay &ly, int dim,
-                        int batch, cudaStream_t s) {
+                        int batch, float *mag, float factor, cudaStream_t s) {
   const size_t pts = dim == 2 ? (size_t)lx.N * lx.N : (size_t)lx.N * lx.N * lx.N;
-  k_c128_to_c64<<<dim3(grid_cap(pts), batch), 256, 0, s>>>(x, lx, y, ly, dim);
+  k_c128_to_c64<<<dim3(grid_cap(pts), batch), 256, 0, s>>>(x, lx, y, ly, dim, mag, factor);
 }
 void launch_c64_to_c128(const float2 *x, const Lay &lx, double2 *y, const Lay &ly, int dim,
                         int batch, cudaStream_t s) {
@@ -272,8 +289,8 @@ void launch_check_inner(SolveState *st, const double *partials,
   else k_check<CHECK_MODE_INNER, false><<<1, 1024, 0, s>>>(st, partials, P, flag, cond, copies, err);
 }
 void launch_check_outer(SolveState *st, const double *partials,
-                        const SolveParams *P, int *flag, cudaStream_t s) {
-  k_check_outer<<<1, 1024, 0, s>>>(st, partials, P, flag);
+                        const SolveParams *P, int *flag, float *mag, cudaStream_t s) {
+  k_check_outer<<<1, 1024, 0, s>>>(st, partials, P, flag, mag);
 }
 void launch_finish(const SolveState *st, const double2 *src, const Lay &ls, double2 *dst,
                    const Lay &ld, int dim, int batch, cudaStream_t s) {
