@@ -374,14 +374,25 @@ template <typename R> Gm2dLevel<R> gm2d_level(hh_handle *h, int l, int dir) {
   g.w.parts2 = h->gm2_parts2;
   return g;
 }
-// The split is that of the handle's batch capacity (at most 16), so that the
-// stop test's number of partial sums does not depend on the call.
-template <typename R> Gm2dPlan gm2d_plan_of(const hh_handle *h, int l, bool restrict_) {
-  return gm2d_plan<R>(h->lv[l].N, h->opt.gmres_m, tune_batch(h), h->sms, restrict_);
+// The split is that of the call's right-hand sides, not of the handle's capacity: one
+// right-hand side on a handle for 16 took as long as 16 (complex128 at 1023^2: 3288 us a
+// cycle instead of 1720, 127^3 1181 instead of 377).  More than 16 share 16's.
+constexpr int kPlanBatch = 16;
+template <typename R> Gm2dPlan gm2d_plan_of(const hh_handle *h, int l, bool restrict_, int batch) {
+  return gm2d_plan<R>(h->lv[l].N, h->opt.gmres_m, std::min(batch, kPlanBatch), h->sms, restrict_);
 }
-
-Gm3dPlan gm3d_plan_of(const hh_handle *h, int l) {
-  return gm3d_plan(h->lv[l].N, tune_batch(h), h->sms);
+Gm3dPlan gm3d_plan_of(const hh_handle *h, int l, int batch) {
+  return gm3d_plan(h->lv[l].N, std::min(batch, kPlanBatch), h->sms, h->opt.precision == HH_FP64);
+}
+// Blocks per right-hand side of a step's sums on level l.
+int gm_parts(const hh_handle *h, int l, int batch) {
+  if (h->dim == 3) return gm3d_plan_of(h, l, batch).blocks;
+  return h->opt.precision == HH_FP64 ? gm2d_plan_of<double>(h, l, true, batch).blocks
+                                     : gm2d_plan_of<float>(h, l, true, batch).blocks;
+}
+// Partial sums per right-hand side of the stop test.
+int nparts_of(const hh_handle *h, int batch) {
+  return h->opt.smoother == HH_SMOOTH_GMRES ? gm_parts(h, 0, batch) : h->nparts;
 }
 
 // One GMRES step on level l: u_out = in + z; restrict_: the restricted residual of
@@ -393,7 +404,7 @@ void enqueue_gm_step(hh_handle *h, int l, int dir, const Gm2dIn<R> &in, typename
   const Gm2dLevel<R> g = gm2d_level<R>(h, l, dir);
   const int m = h->opt.gmres_m;
   if (h->dim == 3) {
-    const Gm3dPlan p = gm3d_plan_of(h, l);
+    const Gm3dPlan p = gm3d_plan_of(h, l, batch);
     launch_gm3d_basis<R>(g.K, g.sigma, g.s, h->kconst, m, in, g.w, p, u_out, batch, st,
                          stop_test(check) ? h->partials : nullptr, s);
     if (stop_test(check)) fork_check(h, check, cond, s);
@@ -407,7 +418,7 @@ void enqueue_gm_step(hh_handle *h, int l, int dir, const Gm2dIn<R> &in, typename
                                  cscal<R>(h, l, dir), batch, st, s);
     return;
   }
-  const Gm2dPlan p = gm2d_plan_of<R>(h, l, restrict_);
+  const Gm2dPlan p = gm2d_plan_of<R>(h, l, restrict_, batch);
   launch_gm2d_basis<R>(g.K, g.sigma, g.s, h->kconst, m, in, g.w, p, batch, st,
                        stop_test(check) ? h->partials : nullptr, s);
   if (stop_test(check)) fork_check(h, check, cond, s);
@@ -820,10 +831,10 @@ void refine_dispatch(hh_handle *h, int dir, const double2 *u_in, int u_zero,
   const LevelK<double> K = levelk<double>(h, 0, dir);
   if (h->dim == 2)
     launch_refine<2>(K, u_in, u_zero, e, u_out, h->w64.f[0], h->w32.f[0],
-                     batch, h->st, h->partials, h->nparts, s);
+                     batch, h->st, h->partials, nparts_of(h, batch), s);
   else
     launch_refine<3>(K, u_in, u_zero, e, u_out, h->w64.f[0], h->w32.f[0],
-                     batch, h->st, h->partials, h->nparts, s);
+                     batch, h->st, h->partials, nparts_of(h, batch), s);
 }
 
 // Loop control: a WHILE graph node (default), or HH_LOOP=host in the
@@ -967,7 +978,7 @@ hh_status set_params(hh_handle *h, int batch, double tol, cudaStream_t s) {
   P.max_cycles = h->opt.max_cycles;
   P.max_inner = h->opt.max_inner;
   P.batch = batch;
-  P.nparts = h->nparts;
+  P.nparts = nparts_of(h, batch);
   HH_CK(cudaMemcpyAsync(h->params, h->params_h, sizeof(SolveParams),
                         cudaMemcpyHostToDevice, s));
   return HH_OK;
@@ -1014,7 +1025,7 @@ hh_status solve_core(hh_handle *h, int dir, const double2 *rhs,
   // that gave up in an earlier solve leaves a partial count behind)
   if (h->pbar) HH_CK(cudaMemsetAsync(h->pbar, 0, 2 * sizeof(unsigned int), s));
   h->fixed_kernels = 3;   // norm of f, state init, final copy
-  launch_norm2(h->w64.f[0], (size_t)l0.S, batch, h->partials, h->nparts, s);
+  launch_norm2(h->w64.f[0], (size_t)l0.S, batch, h->partials, nparts_of(h, batch), s);
   launch_state_init(h->st, h->partials, h->params, h->flag, s);
 
   if (h->opt.precision == HH_FP64) {
@@ -1090,9 +1101,9 @@ void time_one(hh_handle *h, int kernel, int level, int batch, cudaStream_t s) {
   const bool tiled = !two && !pointwise3d(h);   // the kernels the 3-D cycle runs
   if (kernel == 0) {
     double *parts = level == 0 ? h->partials : nullptr;
-    if (two) launch_smooth<R, 2>(K, W.u_post[level], ZERO_NONE, W.f[level], W.u_pre[level], om, batch, nullptr, parts, h->nparts, s);
+    if (two) launch_smooth<R, 2>(K, W.u_post[level], ZERO_NONE, W.f[level], W.u_pre[level], om, batch, nullptr, parts, nparts_of(h, batch), s);
     else if (tiled) launch_smooth3d<R>(K, W.u_post[level], ZERO_NONE, W.f[level], W.u_pre[level], om, batch, nullptr, parts, s);
-    else launch_smooth<R, 3>(K, W.u_post[level], ZERO_NONE, W.f[level], W.u_pre[level], om, batch, nullptr, parts, h->nparts, s);
+    else launch_smooth<R, 3>(K, W.u_post[level], ZERO_NONE, W.f[level], W.u_pre[level], om, batch, nullptr, parts, nparts_of(h, batch), s);
   } else if (kernel == 1) {
     const Lay lc = lay_of(h, level + 1);
     if (two) launch_resid_restrict<R, 2>(K, W.u_pre[level], W.f[level], W.f[level + 1], lc, cscal<R>(h, level, 0), batch, nullptr, s);
@@ -1975,11 +1986,10 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     // stored basis per level, in the cycle's precision: 3-D q_0..q_2, 2-D only in
     // complex128, and complex128 X q_{m-1} as well (zero padding columns)
     HH_CK(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device));
-    const int tb = tune_batch(h);
-    size_t parts = dim == 2 ? gm2d_max_parts(tb, h->sms) : 0;
+    size_t parts = 0;   // partial matrices of the largest call
     for (int l = 0; l + 1 < L; ++l) {
       const size_t np = (size_t)h->lv[l].S * B;
-      if (dim == 3) parts = std::max<size_t>(parts, gm3d_plan_of(h, l).blocks);
+      for (int b = 1; b <= B; ++b) parts = std::max(parts, (size_t)b * gm_parts(h, l, b));
       if (h->opt.precision == HH_FP64) {
         HH_TRY(dev_alloc_n(h, &h->w64.gq[l], 4 * np));
         HH_CK(cudaMemsetAsync(h->w64.gq[l], 0, 4 * np * sizeof(double2), s));
@@ -1989,7 +1999,7 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
       }
     }
     double *q = nullptr;   // 16 sums per block: FP64, or FP32 pairs
-    HH_TRY(dev_alloc_n(h, &q, 16 * parts * B));
+    HH_TRY(dev_alloc_n(h, &q, 16 * parts));
     h->gm2_parts = q;
     HH_TRY(dev_alloc_n(h, &h->gm2_zero, (size_t)B));
     HH_CK(cudaMemsetAsync(h->gm2_zero, 0, (size_t)B * sizeof(int), s));
@@ -2043,8 +2053,7 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
     h->parts_cap = std::max(h->parts_cap, tile_parts(v, h->lv[0].N));
   if (dim == 3) h->parts_cap = std::max(h->parts_cap, tiles3d(h->lv[0].N));
   if (h->opt.smoother == HH_SMOOTH_GMRES)
-    h->parts_cap = std::max(h->parts_cap, dim == 2 ? gm2d_max_parts(tune_batch(h), h->sms)
-                                                   : gm3d_plan_of(h, 0).blocks);
+    for (int b = 1; b <= B; ++b) h->parts_cap = std::max(h->parts_cap, gm_parts(h, 0, b));
   HH_TRY(dev_alloc_n(h, &h->partials, (size_t)h->parts_cap * B));
   HH_TRY(dev_alloc_n(h, &h->err, 1));
   HH_CK(cudaMemsetAsync(h->err, 0, sizeof(int), s));
@@ -2120,11 +2129,6 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   // the 3-D weighted-Jacobi cycle's level-0 sweep writes one partial sum per box
   if (dim == 3 && h->opt.smoother == HH_SMOOTH_JACOBI && !pointwise3d(h))
     h->nparts = tiles3d(h->lv[0].N);
-  // the GMRES cycle's first level-0 step writes one partial sum per block
-  if (h->opt.smoother == HH_SMOOTH_GMRES)
-    h->nparts = dim == 3 ? gm3d_plan_of(h, 0).blocks
-                         : (h->opt.precision == HH_FP64 ? gm2d_plan_of<double>(h, 0, true)
-                                                        : gm2d_plan_of<float>(h, 0, true)).blocks;
   return HH_OK;
 }
 
@@ -3224,10 +3228,10 @@ hh_status hh_time_kernel(hh_handle *h, int kernel, int level, int batch,
       const LevelK<double> K = levelk<double>(h, 0, 0);
       if (h->dim == 2)
         launch_refine<2>(K, h->u64[0], 0, h->w32.u_post[0], h->u64[1], h->w64.f[0], h->w32.f[0],
-                         batch, nullptr, h->partials, h->nparts, s);
+                         batch, nullptr, h->partials, nparts_of(h, batch), s);
       else
         launch_refine<3>(K, h->u64[0], 0, h->w32.u_post[0], h->u64[1], h->w64.f[0], h->w32.f[0],
-                         batch, nullptr, h->partials, h->nparts, s);
+                         batch, nullptr, h->partials, nparts_of(h, batch), s);
       return;
     }
     if (h->opt.precision == HH_FP64)

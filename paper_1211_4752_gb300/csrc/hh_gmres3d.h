@@ -13,7 +13,7 @@ struct Gm3dPlan {
   int planes, blocks;
   int ublocks;
 };
-Gm3dPlan gm3d_plan(int N, int batch, int sms);
+Gm3dPlan gm3d_plan(int N, int batch, int sms, bool fp64);
 
 // One step: basis kernels (q_0 .. q_{m-1} into w.q, the partial Gram matrices),
 // check: per-block |f - A w|^2 for the stop test, or null), and the update
