@@ -678,7 +678,7 @@ void enqueue_tail(hh_handle *h, int dir, int batch, const SolveState *st, cudaSt
     }
   }
   if constexpr (std::is_same<R, double>::value) {
-    if (h->tailop64[dir] && batch <= kTailOp64Batch) {
+    if (h->tailop64[dir] && batch <= tail_op64_batch(h->lv[h->tail0].N)) {
       const LevelHost &v = h->lv[h->tail0];
       launch_tail_apply64(h->tailop64[dir], v.N, v.P, (int)v.S, h->w64.f[h->tail0],
                           h->w64.u_post[h->tail0], batch, st, s);

@@ -307,9 +307,12 @@ void launch_check_list(const CheckList &a, cudaStream_t s);
 void launch_unit_rhs(double2 *F, int N, int P, int S, cudaStream_t s);
 template <typename R>
 void launch_tail_gather(const double2 *U, typename Cx<R>::T *T, int N, int P, int S, cudaStream_t s);
-// complex128 tail operator, for batches of at most kTailOp64Batch right-hand sides:
-// 7.5 us each, against 60 us for the tail kernel whatever the batch
-constexpr int kTailOp64Batch = 6;
+// Right-hand sides up to which the complex128 tail from N points per axis runs as one
+// dense operator: about 9 us each, against the tail kernel's 15 us (N = 7), 26 us (15) and
+// 60 us (31) whatever the batch.  A cycle with the operator and with the kernel (us):
+// 15^2 grid 33 / 39 for one right-hand side, 41 / 39 for two; 31^2 45 / 53 for two,
+// 53 / 53 for three; 63^2 82 / 88 for five, 92 / 88 for six; 127^2 110 / 119, 135 / 119.
+inline int tail_op64_batch(int N) { return N <= 7 ? 1 : (N <= 15 ? 2 : 5); }
 void launch_tail_apply64(const double2 *T, int N, int P, int S, const double2 *f, double2 *u,
                          int batch, const SolveState *st, cudaStream_t s);
 void launch_tail_apply(const float2 *T, int N, int P, int S, const float2 *f, float2 *u,
