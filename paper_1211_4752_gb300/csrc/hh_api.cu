@@ -2072,7 +2072,7 @@ hh_status setup_impl(hh_handle *h, const double *k2_dev, double k2_const,
   double *krange_d = nullptr, krange[2] = {k2_const, k2_const};
   const bool range = h->opt.smoother == HH_SMOOTH_GMRES && k2_dev;
   if (range) {
-    HH_TRY(dev_alloc_n(h, &krange_d, 2));
+    HH_TRY(dev_alloc_n(h, &krange_d, 2 + 2 * kK2RangeBlocks));
     const LevelHost &v = h->lv[0];
     launch_k2_range(v.k2_64, v.N, v.P, rows_of(h, 0), krange_d, s);
     HH_CK(cudaMemcpyAsync(krange, krange_d, sizeof(krange), cudaMemcpyDeviceToHost, s));

@@ -80,7 +80,8 @@ template <> void launch_gm2d_update<double>(const LevelK<double> &, double2, dou
                                             const Gm2dPlan &, double2 *, double2 *, double2,
                                             const Lay &, int, const SolveState *, cudaStream_t);
 
-// (min, max) of the k^2 field of level 0 into out[0..1] (one block).
+// (min, max) of the k^2 field of level 0 into out[0..1]; out: 2 + 2 kK2RangeBlocks.
+constexpr int kK2RangeBlocks = 304;
 void launch_k2_range(const double *k2, int N, int P, size_t rows, double *out, cudaStream_t s);
 
 }  // namespace hh

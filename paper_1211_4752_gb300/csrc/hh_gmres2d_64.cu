@@ -461,12 +461,13 @@ bool use_tiles(int N, int batch) {
 }
 constexpr int kMaxRows = 32;   // rows of a large tile
 
-__global__ void __launch_bounds__(1024) k_k2_range(const double *k2, int N, int P, size_t rows,
-                                                   double *out) {
-  __shared__ double lo[32], hi[32];
+// (min, max) over the rows a block takes, into part[2 blockIdx.x ..].
+__global__ void __launch_bounds__(256) k_k2_range(const double *k2, int N, int P, size_t rows, double *part) {
+  __shared__ double lo[8], hi[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double a = k2[0], c = k2[0];
-  for (size_t r = threadIdx.x >> 5; r < rows; r += 32)
-    for (int x = threadIdx.x & 31; x < N; x += 32) {
+  for (size_t r = (size_t)blockIdx.x * 8 + warp; r < rows; r += (size_t)gridDim.x * 8)
+    for (int x = lane; x < N; x += 32) {
       const double v = k2[r * P + x];
       a = fmin(a, v);
       c = fmax(c, v);
@@ -475,18 +476,18 @@ __global__ void __launch_bounds__(1024) k_k2_range(const double *k2, int N, int 
     a = fmin(a, __shfl_xor_sync(0xffffffffu, a, o));
     c = fmax(c, __shfl_xor_sync(0xffffffffu, c, o));
   }
-  if ((threadIdx.x & 31) == 0) {
-    lo[threadIdx.x >> 5] = a;
-    hi[threadIdx.x >> 5] = c;
+  if (lane == 0) {
+    lo[warp] = a;
+    hi[warp] = c;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int i = 1; i < 32; ++i) {
+    for (int i = 1; i < 8; ++i) {
       lo[0] = fmin(lo[0], lo[i]);
       hi[0] = fmax(hi[0], hi[i]);
     }
-    out[0] = lo[0];
-    out[1] = hi[0];
+    part[2 * blockIdx.x] = lo[0];
+    part[2 * blockIdx.x + 1] = hi[0];
   }
 }
 
@@ -496,8 +497,12 @@ __global__ void __launch_bounds__(1024) k_k2_range(const double *k2, int N, int 
 // over the batch (every block of the update kernel adds them all).
 int gm2d_max_parts(int batch, int sms) { return std::max(256, 2 * sms / std::max(1, batch)); }
 
+// Blocks of eight rows, and one over their results: min(all) and max(all) of the pairs.
+// (One block for the whole field took 10 ms at 4095^2.)
 void launch_k2_range(const double *k2, int N, int P, size_t rows, double *out, cudaStream_t s) {
-  k_k2_range<<<1, 1024, 0, s>>>(k2, N, P, rows, out);
+  const int blocks = (int)std::min<size_t>(kK2RangeBlocks, (rows + 7) / 8);
+  k_k2_range<<<blocks, 256, 0, s>>>(k2, N, P, rows, out + 2);
+  k_k2_range<<<1, 256, 0, s>>>(out + 2, 2 * blocks, 2 * blocks, 1, out);
 }
 
 // Rows of a tile: as many as leave about two tiles per SM over the batch (tall
