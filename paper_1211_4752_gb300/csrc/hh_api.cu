@@ -1794,7 +1794,7 @@ template <typename R> hh_status setup_gmres_tail(hh_handle *h) {
     a.nu2 = h->opt.nu2;
     auto pts = [&](int n) { return (size_t)(n + 1) * (h->dim == 2 ? n : n * n); };   // pitched
     size_t c = 0, r = 0;
-    for (int q = 0; q < 3; ++q) { a.offQ[q] = (int)c; c += pts(h->lv[t0].N); }
+    for (int q = 0; q < (sizeof(R) == 8 ? 4 : 3); ++q) { a.offQ[q] = (int)c; c += pts(h->lv[t0].N); }
     for (int i = 0; i < a.nl; ++i) {
       const int l = t0 + i;
       GmTailLevel<R> &g = a.lv[i];

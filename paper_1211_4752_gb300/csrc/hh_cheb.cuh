@@ -33,9 +33,6 @@
 namespace hh {
 
 constexpr int kGramPairMaxN = 256;   // complex64: paired sums up to this N (2-D)
-// complex128: a step with a smaller pivot (relative to its diagonal entry) gets
-// one step of refinement
-constexpr double kPivotOk = 1e-3;
 
 // ---- accumulators ----------------------------------------------------------
 template <typename R, bool PAIR> struct GramAcc;
@@ -253,16 +250,19 @@ struct Fp64 {
 template <typename R> struct SolveNum { using T = PairF; };
 template <> struct SolveNum<double> { using T = Fp64; };
 
-// Coefficients of one step's update, z_j = s y_j, in the vectors' precision, and
-// the smallest pivot relative to its diagonal entry.
+// Coefficients of one step's update, z_j = s y_j, in the vectors' precision;
+// complex128: and the inverse of N, for the correction of y (solve_correction).
 template <typename R> struct StepCoef {
   typename Cx<R>::T z[3];
-  R pivot;
+};
+template <> struct StepCoef<double> {
+  double2 z[3];
+  double2 inv[3][3];
 };
 
 // Solve N y = b from the Gram sums G (NQP entries, shared memory) by
 // Gauss-Jordan elimination, one warp, lane 4 i + j holding entry (i, j) of
-// [N | b], and store the step's coefficients.  N is Hermitian and positive
+// [N | b], and store the step's coefficients (complex128: the inverse grows in N's place).  N is Hermitian and positive
 // semidefinite; a pivot that is at most tol times its diagonal entry marks a
 // vector in the span of the earlier ones: its coefficient is zero (the Krylov
 // space has ended).  Called by the 32 lanes of one warp.
@@ -285,15 +285,16 @@ __device__ __forceinline__ void gram_solve(const typename GramSum<R>::T *G, R s,
     }
   }
   const T diag = ax;
-  R pivot = R(1);
 #pragma unroll
   for (int k = 0; k < M; ++k) {
     const T pk = ax.shfl(5 * k), dk = diag.shfl(5 * k), rp = pk.pivot_rcp(dk, tol);
-    if (sizeof(R) == 8 && rp.lead() > R(0) && R(pk.lead()) < pivot * R(dk.lead()))
-      pivot = R(pk.lead()) / R(dk.lead());
     // row k scaled, and this row's entry of column k
-    const T kx = ax.shfl(4 * k + j).mul(rp), ky = ay.shfl(4 * k + j).mul(rp);
+    T kx = ax.shfl(4 * k + j).mul(rp), ky = ay.shfl(4 * k + j).mul(rp);
     const T lx = ax.shfl(4 * i + k), ly = ay.shfl(4 * i + k);
+    if (sizeof(R) == 8 && j == k) {   // the inverse's column, from the unit matrix
+      kx = rp;
+      ax = ay = ky = T::zero();
+    }
     if (i == k) {
       ax = kx;
       ay = ky;
@@ -306,7 +307,38 @@ __device__ __forceinline__ void gram_solve(const typename GramSum<R>::T *G, R s,
     out->z[i].x = R(ax.lead()) * s;
     out->z[i].y = R(ay.lead()) * s;
   }
-  if (lane == 0) out->pivot = pivot;
+  if constexpr (sizeof(R) == 8) {
+    if (i < M && j < M) out->inv[i][j] = make_double2(ax.lead(), ay.lead());
+  }
+}
+
+// complex128: y from the normal equations alone loses digits by N's condition (a cycle
+// against quad precision 2e-15 to 7e-15 where an orthogonalised basis gave 0.8e-15, a step
+// on smooth residuals 1e-13).  One correction restores them (corrected seminormal
+// equations, Bjorck 1987): d_i = <a_i, r - sum y_j a_j> from the vectors, y += N^-1 d.
+// Lanes 0 .. M - 1 of a warp; d: real and imaginary parts (shared memory).
+template <int M>
+__device__ __forceinline__ void solve_correction(const double *d, double s, StepCoef<double> *c) {
+  const int i = threadIdx.x & 31;
+  if (i >= M) return;
+  double2 y = czero<double2>();
+#pragma unroll
+  for (int j = 0; j < M; ++j) y = cfma(c->inv[i][j], make_double2(d[2 * j], d[2 * j + 1]), y);
+  c->z[i] = cadd(c->z[i], cscale(y, s));
+}
+// a point's part of d (acc[2 j], acc[2 j + 1]) from a_j and r
+template <int M>
+__device__ __forceinline__ void correction_point(GramAcc<double, false> (&acc)[8], const double2 (&a)[M],
+                                                 const double2 (&y)[M], double2 r) {
+#pragma unroll
+  for (int j = 0; j < M; ++j) r = cfnma(y[j], a[j], r);
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    acc[2 * j].mac(a[j].x, r.x);
+    acc[2 * j].mac(a[j].y, r.y);
+    acc[2 * j + 1].mac(a[j].x, r.y);
+    acc[2 * j + 1].mac(-a[j].y, r.x);
+  }
 }
 
 // Pivot tolerance: above the rounding of the sums (1e-14 paired, 1e-8 plain

@@ -59,7 +59,7 @@ template <typename R, int DIM, int M>
 __device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s, R g,
                              typename Cx<R>::T *U, const typename Cx<R>::T *F,
                              typename Cx<R>::T *Q0, typename Cx<R>::T *Q1, typename Cx<R>::T *Q2,
-                             bool zero, bool res,
+                             typename Cx<R>::T *Q3, bool zero, bool res,
                              typename GramSum<R>::T *sums, StepCoef<R> *sc) {
   using C = typename Cx<R>::T;
   constexpr bool PAIR = sizeof(R) == 4;
@@ -110,6 +110,7 @@ __device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s, R
     if (M >= 2) v[1] = cfma(t, v[0], Q1[p]);
     if (M == 3) v[M - 1] = cfma(t, Q1[p], cscale(cadd(qc, v[0]), R(0.5)));
     v[M] = cfma(t, qc, xl);
+    if (sizeof(R) == 8) Q3[p] = xl;   // (read by this thread alone)
     gram_point<R, M, PAIR>(acc, v);
   });
   constexpr int SH = NQP == 16 ? 1 : 3;
@@ -133,51 +134,37 @@ __device__ void tail_gm_step(const LevelK<R> &K, typename Cx<R>::T sigma, R s, R
     gram_solve<R, M>(sums, sizeof(R) == 4 ? s * (R)gram_rcp((float)g) : s, gram_tol<R>(PAIR), sc);
   }
   __syncthreads();
-  if constexpr (sizeof(R) == 8) {
-    // small pivot: one step of refinement (see k_gm2d_coef, hh_gmres2d_64.cu)
-    if (sc->pivot < kPivotOk) {
-      using A = GramAcc<double, false>;
-      A cor[8];
+  if constexpr (sizeof(R) == 8) {   // the coefficients' correction (solve_correction)
+    using A = GramAcc<double, false>;
+    A cor[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) cor[i].zero();
-      double2 yc[M];
+    for (int i = 0; i < 8; ++i) cor[i].zero();
+    double2 yc[M];
 #pragma unroll
-      for (int j = 0; j < M; ++j) yc[j] = cscale(sc->z[j], 1.0 / s);
-      tail_points<DIM>(N, [&](int p, int x, int y, int z) {
-        C qc, a[M];
-        const C xl = X(M == 1 ? Q0 : (M == 2 ? Q1 : Q2), x, y, z, qc);
-        if (M >= 2) a[0] = cfma(t, Q0[p], Q1[p]);
-        if (M == 3) a[1 % M] = cfma(t, Q1[p], cscale(cadd(qc, Q0[p]), 0.5));
-        a[M - 1] = cfma(t, qc, xl);
-        C r = Q0[p];
-#pragma unroll
-        for (int j = 0; j < M; ++j) r = csub(r, cmul(yc[j], a[j]));
-#pragma unroll
-        for (int j = 0; j < M; ++j) {
-          cor[2 * j].mac(a[j].x, r.x);
-          cor[2 * j].mac(a[j].y, r.y);
-          cor[2 * j + 1].mac(a[j].x, r.y);
-          cor[2 * j + 1].mac(-a[j].y, r.x);
-        }
-      });
-      const A v = gram_warp_sum<A, 8>(cor);
-      double *corr = sums + 16;   // (the warps' sums are used up)
-      if ((lane & 3) == 0) corr[warp * 8 + (lane >> 2)] = v.h;
-      __syncthreads();
-      if (warp == 0) {
-        double q = 0.0;
-        if (lane < 8)
-          for (int w = 0; w < TB / 32; ++w) q += corr[w * 8 + lane];
-        if (lane < 2 * M) sums[Gram<M>::pair(0, lane / 2 + 1) + (lane & 1)] = (lane & 1) ? -q : q;
-        __syncwarp();
-        const C z0 = lane < 3 ? sc->z[lane] : czero<C>();
-        __syncwarp();
-        gram_solve<R, M>(sums, s, gram_tol<R>(PAIR), sc);
-        __syncwarp();
-        if (lane < 3) sc->z[lane] = cadd(z0, sc->z[lane]);
-      }
-      __syncthreads();
+    for (int j = 0; j < M; ++j) yc[j] = cscale(sc->z[j], 1.0 / s);
+    tail_points<DIM>(N, [&](int p, int, int, int) {
+      C a[M];
+      const C qc = (M == 1 ? Q0 : (M == 2 ? Q1 : Q2))[p], xl = Q3[p];
+      if (M >= 2) a[0] = cfma(t, Q0[p], Q1[p]);
+      if (M == 3) a[1 % M] = cfma(t, Q1[p], cscale(cadd(qc, Q0[p]), 0.5));
+      a[M - 1] = cfma(t, qc, xl);
+      correction_point<M>(cor, a, yc, Q0[p]);
+    });
+    const A v = gram_warp_sum<A, 8>(cor);
+    if ((lane & 3) == 0) sums[warp * 8 + (lane >> 2)] = v.h;
+    __syncthreads();
+    if (warp == 0) {
+      const int nw = min(TB / 32, ((int)K.S + 31) / 32);   // (as above)
+      double d = 0.0;
+      for (int w = lane >> 3; w < nw; w += 4) d += sums[w * 8 + (lane & 7)];
+      d += __shfl_xor_sync(0xffffffffu, d, 8);
+      d += __shfl_xor_sync(0xffffffffu, d, 16);
+      __syncwarp();
+      if (lane < 8) sums[lane] = d;
+      __syncwarp();
+      solve_correction<M>(sums, s, sc);
     }
+    __syncthreads();
   }
   tail_points<DIM>(N, [&](int p, int, int, int) {
     C v = zero ? czero<C>() : U[p];
@@ -208,10 +195,10 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
   R *km = reinterpret_cast<R *>(smem_raw + A.kbase);
   double2 *sinv = reinterpret_cast<double2 *>(smem_raw + A.invbase);
   const int mm = A.mm;
-  // (complex128: room for the refinement's sums behind the Gram matrix)
-  __shared__ typename GramSum<R>::T sums[sizeof(R) == 8 ? 16 + (TB / 32) * 16 : (TB / 32) * Gram<M>::NQP];
+  __shared__ typename GramSum<R>::T sums[(TB / 32) * 16];
   __shared__ StepCoef<R> sc;
   C *const Q0 = cm + A.offQ[0], *const Q1 = cm + A.offQ[1], *const Q2 = cm + A.offQ[2];
+  C *const Q3 = cm + A.offQ[sizeof(R) == 8 ? 3 : 2];
   // every level's tables and k^2 and the coarsest inverse, which no kernel writes: staged
   // before the dependency wait
   for (int i = 0; i < A.nl; ++i) {
@@ -241,7 +228,7 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
     C *U = cm + A.lv[i].offU;
     const C *F = cm + A.lv[i].offF;
     for (int s = 0; s < A.nu1; ++s)
-      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, g, U, F, Q0, Q1, Q2, s == 0,
+      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, g, U, F, Q0, Q1, Q2, Q3, s == 0,
                               s == A.nu1 - 1, sums, &sc);
     {
       const C *r = Q0;
@@ -306,7 +293,7 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
     });
     __syncthreads();
     for (int s = 0; s < A.nu2; ++s)
-      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, g, U, F, Q0, Q1, Q2, false, false,
+      tail_gm_step<R, DIM, M>(K, A.lv[i].sigma, A.lv[i].s, g, U, F, Q0, Q1, Q2, Q3, false, false,
                               sums, &sc);
   }
   {
@@ -319,14 +306,14 @@ __global__ void __launch_bounds__(TB) k_gm_tail(const __grid_constant__ GmTailAr
 
 }  // namespace
 
-// Shared memory of the tail (layout of setup_gmres_tail): q_0..q_2 of the first
-// level, per level iterate, right-hand side, tables and k^2 (rows
+// Shared memory of the tail (layout of setup_gmres_tail): q_0..q_2 (complex128: and
+// X q_{m-1}) of the first level, per level iterate, right-hand side, tables and k^2 (rows
 // of pitch N + 1), the coarsest inverse.
 static size_t tail_pts(int dim, int N) { return (size_t)(N + 1) * (dim == 2 ? N : N * N); }
 template <typename R, int DIM> size_t gmres_tail_smem(const int *N, int nl, int m) {
   (void)m;
   using C = typename Cx<R>::T;
-  size_t c = 3 * tail_pts(DIM, N[0]);
+  size_t c = (sizeof(R) == 8 ? 4 : 3) * tail_pts(DIM, N[0]);
   size_t r = 0;
   for (int i = 0; i < nl; ++i) {
     c += 2 * tail_pts(DIM, N[i]) + 3 * DIM * (size_t)N[i];

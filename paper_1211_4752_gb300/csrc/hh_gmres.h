@@ -26,7 +26,7 @@ template <typename R> struct GmTailLevel {
 template <typename R> struct GmTailArgs {
   int nl, m, nu1, nu2;
   GmTailLevel<R> lv[kGmTailMax];
-  int offQ[3];                 // q_0..q_2 (sized for level t0)
+  int offQ[4];                 // q_0..q_2, complex128: X q_{m-1} (sized for level t0)
   int kbase, invbase, smem_bytes;
   const typename Cx<R>::T *f;  // right-hand side of level t0 (library layout lay)
   typename Cx<R>::T *u;        // its correction

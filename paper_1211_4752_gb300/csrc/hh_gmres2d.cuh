@@ -110,29 +110,26 @@ __device__ __forceinline__ void step_coef(const typename GramSum<R>::T *parts, i
   __syncthreads();
 }
 
-// complex128: the coefficients that k_gm2d_coef stored, with its correction where
-// one follows (nb: its blocks).  One warp; sums: 16 slots.
+// complex128: the coefficients that k_gm2d_coef stored, with the correction from its nb
+// blocks' sums.  One warp; sums: 8 slots.
 template <int M>
 __device__ __forceinline__ void read_coef(const Gm2dWork<double> &wk, int b, int nb, double s,
-                                          double tol, double *sums, StepCoef<double> *out) {
+                                          double *sums, StepCoef<double> *out) {
   const int lane = threadIdx.x & 31;
-  const double *c = wk.coef + (size_t)b * kGm2dCoef;
-  if (lane < 3) out->z[lane] = make_double2(c[2 * lane], c[2 * lane + 1]);
-  if (c[6] == 0.0) return;
-  // right-hand side <a_i, r - sum y_j a_j> in the place of <a_i, r>
-  double t = 0.0;
-  for (int i = lane >> 3; i < nb; i += 4) t += wk.parts2[((size_t)b * kGm2dCorr + i) * 8 + (lane & 7)];
-  t += __shfl_xor_sync(0xffffffffu, t, 8);
-  t += __shfl_xor_sync(0xffffffffu, t, 16);
-  if (lane < Gram<M>::NQP) sums[lane] = c[8 + lane];
+  static_assert(sizeof(StepCoef<double>) == kGm2dCoef * sizeof(double), "coefficients");
+  if (lane < kGm2dCoef) reinterpret_cast<double *>(out)[lane] = wk.coef[(size_t)b * kGm2dCoef + lane];
+  const double *p = wk.parts2 + (size_t)b * kGm2dCorr * 8 + (lane & 7);
+  double t[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = lane >> 3; i < nb; i += 16)   // four loads in flight
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (i + 4 * r < nb) t[r] += p[(size_t)(i + 4 * r) * 8];
+  double d = (t[0] + t[1]) + (t[2] + t[3]);
+  d += __shfl_xor_sync(0xffffffffu, d, 8);
+  d += __shfl_xor_sync(0xffffffffu, d, 16);
+  if (lane < 8) sums[lane] = d;
   __syncwarp();
-  if (lane < 2 * M) sums[Gram<M>::pair(0, lane / 2 + 1) + (lane & 1)] = (lane & 1) ? -t : t;
-  __syncwarp();
-  const double2 z = lane < 3 ? out->z[lane] : czero<double2>();
-  __syncwarp();
-  gram_solve<double, M>(sums, s, tol, out);
-  __syncwarp();
-  if (lane < 3) out->z[lane] = cadd(z, out->z[lane]);
+  solve_correction<M>(sums, s, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -326,7 +323,7 @@ k_gm2d_update_tile(LevelK<R> L, typename Cx<R>::T sigma, R s, Gm2dIn<R> in, Gm2d
       solve_warp<R, M>(sums, NT / 32, s, tol, &sc);
       if (wk.track && blockIdx.x == 0 && tid == NC) gram_estimate(wk.mag, b, sums[0], wk.g[b]);
     }
-    else read_coef<M>(wk, b, nparts, s, tol, sums, &sc);
+    else read_coef<M>(wk, b, nparts, s, sums, &sc);
   }
   else tile_basis<R, M, E>(op, fv, sw, sq, sigma, s, R(1), tx, ty, mine, 1, NC);
   __syncthreads();

@@ -38,8 +38,8 @@ template <typename R> struct Gm2dWork {
   double *coef;                 // the solved coefficients ([b][kGm2dCoef]) and the
   double *parts2;               // sums of their correction ([b][block][8])
 };
-constexpr int kGm2dCoef = 32;   // z_0..z_2, whether a correction follows, Gram matrix (16)
-constexpr int kGm2dCorr = 128;  // blocks of the correction's sums at most
+constexpr int kGm2dCoef = 24;   // StepCoef<double>: z_0..z_2, the inverse of N
+constexpr int kGm2dCorr = 152;  // blocks of the correction's sums at most
 
 template <typename R> cudaError_t init_gm2d();   // once per complex128 handle
 template <typename R> Gm2dPlan gm2d_plan(int N, int m, int batch, int sms, bool restrict_);

@@ -316,44 +316,36 @@ __device__ __forceinline__ void restrict_body(const TileCtx<R, MODE> &t, ColumnO
 }
 
 // The step's coefficients from the partial Gram matrices, for the update kernel
-// (every block of this kernel adds and solves; block 0 stores).  Where a pivot is
-// below kPivotOk the normal equations lose digits that matter over hundreds of
-// cycles (an FP64 solve of the 511^2 layered medium followed the oracle's residual
-// history over 400 cycles to 2e-7 instead of 1e-11): then r - sum y_j a_j is formed
-// from the stored vectors and its inner products with the a_j, per block, correct
-// the solution (corrected seminormal equations, Bjorck 1987).
+// (every block of this kernel adds and solves; block 0 stores), and per block the sums of
+// their correction (solve_correction) from the stored vectors.  Bound by the FP64 pipe
+// (about 32 instructions per point): 88 us at 1023^2, 39 at 511^2, 11 on small levels.
 template <int M>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
 k_gm2d_coef(LevelK<double> L, int rows, double2 sigma, double s, Gm2dWork<double> wk, int nparts,
             double tol, const SolveState *st) {
   constexpr int NQP = Gram<M>::NQP;
   using A = GramAcc<double, false>;
-  __shared__ double sums[8 * 16];
+  __shared__ double sums[32 * 16];
   __shared__ StepCoef<double> sc;
   const int b = blockIdx.y;
   griddep_wait();
   griddep_launch_dependents();
   if (!__syncthreads_and(!(st && !st[b].active))) return;
   step_coef<double, M>(wk.parts + (size_t)b * nparts * NQP, nparts, s, tol, sums, &sc);
-  const bool correct = sc.pivot < kPivotOk;
-  if (blockIdx.x == 0) {
-    double *c = wk.coef + (size_t)b * kGm2dCoef;
-    if (threadIdx.x < 3) {
-      c[2 * threadIdx.x] = sc.z[threadIdx.x].x;
-      c[2 * threadIdx.x + 1] = sc.z[threadIdx.x].y;
-    }
-    if (threadIdx.x == 3) c[6] = correct ? 1.0 : 0.0;
-    if (threadIdx.x < NQP) c[8 + threadIdx.x] = sums[threadIdx.x];
-  }
-  if (!correct) return;
-  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x < kGm2dCoef)
+    wk.coef[(size_t)b * kGm2dCoef + threadIdx.x] = reinterpret_cast<const double *>(&sc)[threadIdx.x];
   A acc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i].zero();
   double2 y[M];
 #pragma unroll
-  for (int j = 0; j < M; ++j) y[j] = cscale(sc.z[j], 1.0 / s);
-  const double2 t = cscale(sigma, s);
+  for (int j = 0; j < M; ++j) y[j] = cscale(sc.z[j], (M == 3 && j == 1 ? 0.5 : 1.0) / s);
+  const double2 t = cscale(sigma, s), t2 = cadd(t, t);
+  auto shifted = [](double2 c, double2 q, double2 xq) {   // xq + c q (c: real on the finest level)
+    double2 r = make_double2(fma(c.x, q.x, xq.x), fma(c.x, q.y, xq.y));
+    if (c.y != 0.0) r = make_double2(fma(-c.y, q.y, r.x), fma(c.y, q.x, r.y));
+    return r;
+  };
   const double2 *q = wk.q + (size_t)b * L.S;
   const int N = L.N;
   for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < (unsigned)rows * (unsigned)N; p += gridDim.x * blockDim.x) {
@@ -361,30 +353,23 @@ k_gm2d_coef(LevelK<double> L, int rows, double2 sigma, double s, Gm2dWork<double
     double2 v[M + 1], a[M];
 #pragma unroll
     for (int j = 0; j <= M; ++j) v[j] = q[(size_t)j * wk.qs + o];   // v[M] = X q_{M-1}
-    a[0] = M == 1 ? cfma(t, v[0], v[1]) : cfma(t, v[0], v[1]);
-    if (M == 2) a[M - 1] = cfma(t, v[1], v[M]);
-    if (M == 3) {
-      a[1 % M] = cfma(t, v[1], cscale(cadd(v[2 % (M + 1)], v[0]), 0.5));
-      a[M - 1] = cfma(t, v[M - 1], v[M]);
+    a[0] = shifted(t, v[0], v[1]);
+    if (M == 2) a[M - 1] = shifted(t, v[1], v[M]);
+    if (M == 3) {   // (twice a_1, with half of y_1 and of d_1)
+      a[1 % M] = shifted(t2, v[1], cadd(v[2 % (M + 1)], v[0]));
+      a[M - 1] = shifted(t, v[M - 1], v[M]);
     }
-    double2 r = v[0];
-#pragma unroll
-    for (int j = 0; j < M; ++j) r = csub(r, cmul(y[j], a[j]));
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      acc[2 * j].mac(a[j].x, r.x);
-      acc[2 * j].mac(a[j].y, r.y);
-      acc[2 * j + 1].mac(a[j].x, r.y);
-      acc[2 * j + 1].mac(-a[j].y, r.x);
-    }
+    correction_point<M>(acc, a, y, v[0]);
   }
   const A v = gram_warp_sum<A, 8>(acc);
+  __syncthreads();   // (block 0 has read the coefficients; the Gram sums are used up)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if ((lane & 3) == 0) sums[warp * 8 + (lane >> 2)] = v.h;
   __syncthreads();
   if (threadIdx.x < 8) {
     double r = 0.0;
-    for (int w = 0; w < 8; ++w) r += sums[w * 8 + threadIdx.x];
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sums[w * 8 + threadIdx.x];
+    if (M == 3 && threadIdx.x >> 1 == 1) r *= 0.5;
     wk.parts2[((size_t)b * kGm2dCorr + blockIdx.x) * 8 + threadIdx.x] = r;
   }
 }
@@ -394,11 +379,11 @@ k_gm2d_coef(LevelK<double> L, int rows, double2 sigma, double s, Gm2dWork<double
 template <int M, bool CORR, bool REST>
 __global__ void __launch_bounds__(kTileThreads)
 k_gm2d_update(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<double> in,
-                     Gm2dWork<double> wk, int nparts, double tol, int ty, double2 *u_out,
+                     Gm2dWork<double> wk, int nparts, int ty, double2 *u_out,
                      double2 *fc, double2 cs, Lay lc, const SolveState *st) {
   constexpr int TX = kTX, O = REST ? 1 : 0, XH = REST ? 3 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double sums[16];
+  __shared__ double sums[8];
   __shared__ StepCoef<double> sc;
   const int hb = tile_rows(M, ty);
   double2 *A = reinterpret_cast<double2 *>(smem_raw), *B = A + hb * kTP, *sr = B + 2 * hb * kTP;
@@ -407,7 +392,7 @@ k_gm2d_update(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<doub
   griddep_launch_dependents();
   if (!__syncthreads_and(!(st && !st[b].active))) return;
   const bool zero = wk.zflag[b] != 0;
-  if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, tol, sums, &sc);
+  if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, sums, &sc);
   __syncthreads();
   const double2 *q = wk.q + (size_t)b * L.S;
   u_out += (size_t)b * L.S;
@@ -564,10 +549,15 @@ void launch_gm2d_basis<double>(const LevelK<double> &L, double2 sigma, double s,
 int launch_gm_coef(const LevelK<double> &L, int rows, double2 sigma, double s, int m,
                    const Gm2dWork<double> &w, int nparts, int batch, const SolveState *st,
                    cudaStream_t stream) {
-  const int nb = std::min(kGm2dCorr, (int)(((long long)rows * L.N + 1023) / 1024));
+  // Small levels: a point per thread.  Large ones: 32 warps per SM (with 8 of them 1023^2
+  // took 320 us), blocks on every SM for two right-hand sides or more (the others of a
+  // batch may have stopped; every block adds and solves before its points)
+  const long long pts = (long long)rows * L.N;
+  const int threads = pts < 65536 ? 256 : 1024;
+  const int nb = (int)std::min<long long>((pts + threads - 1) / threads, batch == 1 || threads == 256 ? kGm2dCorr : kGm2dCorr / 2);
   const double tol = gram_tol<double>(false);
   with_m(m, [&](auto mm) {
-    launch_pdl(k_gm2d_coef<decltype(mm)::value>, dim3(nb, batch), dim3(256), 0, stream, L, rows, sigma, s,
+    launch_pdl(k_gm2d_coef<decltype(mm)::value>, dim3(nb, batch), dim3(threads), 0, stream, L, rows, sigma, s,
                w, nparts, tol, st);
   });
   return nb;
@@ -590,7 +580,7 @@ void launch_gm2d_update<double>(const LevelK<double> &L, double2 sigma, double s
                                                               fc, cs, lc, batch, st, stream);
       else
         launch_pdl(k_gm2d_update<M, CORR, REST>, dim3(p.ublocks, batch), dim3(kTileThreads),
-                   tile_smem(M, p.urows), stream, L, sigma, s, kconst, in, w, nb, tol, p.urows,
+                   tile_smem(M, p.urows), stream, L, sigma, s, kconst, in, w, nb, p.urows,
                    u_out, fc, cs, lc, st);
     };
     if (in.e) go(std::true_type(), std::false_type());

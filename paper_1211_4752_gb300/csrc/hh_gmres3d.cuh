@@ -267,7 +267,7 @@ k_gm3d_update(LevelK<R> L, R s, const typename Cx<R>::T *u_in, Gm2dWork<R> wk, i
     step_coef<R, M>(wk.parts + (size_t)b * nparts * NQP, nparts, s * gram_rcp(g), tol, sums, &sc);
     if (wk.track && blockIdx.x == 0 && threadIdx.x == 0) gram_estimate(wk.mag, b, sums[0], g);
   } else {
-    if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, tol, sums, &sc);
+    if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, sums, &sc);
     __syncthreads();
   }
   C z[M];
