@@ -20,12 +20,18 @@
 // levels correct; the cycles' error against FP64 was 2 to 4 times larger.)
 // Against one reduction per Arnoldi step this leaves one per GMRES step.
 //
-// N's condition number is the square of the basis's (1e2 .. 1e5 on the media
-// measured), so complex64 vectors' products are summed as unevaluated pairs of
-// FP32 values (Dekker / Knuth: the product's and the sum's rounding errors are
-// kept in a second FP32 value), which costs no FP64 arithmetic.  On levels of more than kGramPairMaxN points per axis plain FP32
-// sums serve: their rounding errors are independent over > 1e5 short sums and
-// average to 1e-9 of the sum.
+// N's condition number is the square of the basis's (1e2 .. 1e5 on rough residuals, 1e6
+// and more on smooth ones), so complex64 vectors' products are summed as unevaluated pairs
+// of FP32 values (Dekker / Knuth: the product's and the sum's rounding errors are kept in a
+// second FP32 value), which costs no FP64 arithmetic.  On levels of more than
+// kGramPairMaxN points per axis a thread's own sums are plain FP32, folded into a second
+// value every four rows (3-D: eight planes), and pairs from there on: relative errors of
+// 2.7e-10 (511^2), 2.3e-10 (1023^2), 1.3e-10 (2047^2), 6.1e-10 (511^2, 16 right-hand
+// sides) and 1.9e-10 (127^3; 3.6e-10 with 16); without the folds up to 1.3e-9 and 2.5e-9, with FP32
+// warp sums added in FP64 4.4e-10 to 7.2e-10.  What the nearly parallel vectors of a smooth
+// residual lose to their own rounding stays: a complex64 cycle from zero on smooth
+// right-hand sides is 1 to 5 times as far from the exact one as with an orthogonalised
+// basis (the step's residual is the same to 1e-7), on rough ones no further.
 #pragma once
 #include "hh_internal.h"
 #include "hh_complex.cuh"
@@ -41,6 +47,8 @@ template <> struct GramAcc<double, false> {
   __device__ __forceinline__ void zero() { h = 0.0; }
   __device__ __forceinline__ void mac(double a, double b) { h = fma(a, b, h); }
   __device__ __forceinline__ void add(const GramAcc &o) { h += o.h; }
+  __device__ __forceinline__ void fold() {}
+  __device__ __forceinline__ void close() {}
   __device__ __forceinline__ GramAcc shfl_xor(int m) const {
     GramAcc r;
     r.h = __shfl_xor_sync(0xffffffffu, h, m);
@@ -65,6 +73,18 @@ template <bool PAIR> struct GramAcc<float, PAIR> {
     } else {
       h = fmaf(a, b, h);
     }
+  }
+  // plain sums of a thread: h holds a few points', l those folded before (see above)
+  __device__ __forceinline__ void fold() {
+    if (PAIR) return;
+    l = __fadd_rn(l, h);
+    h = 0.f;
+  }
+  __device__ __forceinline__ void close() {   // (h, l) as a pair again
+    if (PAIR) return;
+    const float t = l;
+    l = 0.f;
+    two_sum(t);
   }
   __device__ __forceinline__ void add(const GramAcc &o) {
     l = __fadd_rn(l, o.l);
@@ -341,7 +361,7 @@ __device__ __forceinline__ void correction_point(GramAcc<double, false> (&acc)[8
   }
 }
 
-// Pivot tolerance: above the rounding of the sums (1e-14 paired, 1e-8 plain
+// Pivot tolerance: above the rounding of the sums (1e-14 paired, 1e-9 plain
 // FP32, 1e-16 FP64) and far below the pivots of a proper step.
 template <typename R> __host__ __device__ constexpr double gram_tol(bool pair) {
   return sizeof(R) == 8 ? 1e-14 : (pair ? 1e-12 : 1e-8);

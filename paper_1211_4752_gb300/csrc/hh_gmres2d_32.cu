@@ -243,8 +243,9 @@ template <typename R, int M, int NX, int MODE, bool CORR, bool FROWS = false> st
   }
 
   // rows [y0, y1); rows outside the domain are zero
-  template <typename W0, typename H, typename E>
-  __device__ __forceinline__ void run(int y0, int y1, W0 w0, H hook, E emit) {
+  // (fold: called every four rows)
+  template <typename W0, typename H, typename E, typename D>
+  __device__ __forceinline__ void run(int y0, int y1, W0 w0, H hook, E emit, D fold) {
     const int ys = y0 - NX, T = y1 - y0 + 2 * NX;
     wmax = y1 + NX;
     fmax = y1 - 1 + NX;
@@ -276,6 +277,7 @@ template <typename R, int M, int NX, int MODE, bool CORR, bool FROWS = false> st
       if (t + 1 < T) step<1>(ys + t + 1, w0, hook, emit);
       if (t + 2 < T) step<2>(ys + t + 2, w0, hook, emit);
       if (t + 3 < T) step<3>(ys + t + 3, w0, hook, emit);
+      fold();
     }
   }
 };
@@ -344,6 +346,11 @@ struct MarchWork {
 };
 
 constexpr int kMaxWarps = 16;   // per block: 128 registers per thread
+// Plain sums, folded every four rows, need more: with 128 registers a 1023^2 step took
+// 57.2 us, with 168 and twelve warps 52.4 (four right-hand sides 146 and 138, 511^2 30.2 and
+// 29.2; unfolded, with 128 registers, 55.6, 139 and 29.4).  Where every warp has several
+// items 16 warps are faster all the same: 4095^2 483 us and 514 (unfolded 462).
+constexpr int kPlainWarps = 12;
 
 template <typename R, int M, bool PAIR, int MODE, bool CORR>
 __device__ __forceinline__ void basis_run(const LevelK<R> &L, const Gm2dIn<R> &in,
@@ -368,17 +375,20 @@ __device__ __forceinline__ void basis_run(const LevelK<R> &L, const Gm2dIn<R> &i
     }
     gram_point<R, M, PAIR>(acc, v);
   };
-  m.run(y0, y1, none0, none, emit);
+  m.run(y0, y1, none0, none, emit, [&] {
+#pragma unroll
+    for (int i = 0; i < Gram<M>::NQ; ++i) acc[i].fold();
+  });
 }
 
-template <typename R, int M, bool PAIR, bool CORR>
-__global__ void __launch_bounds__(32 * kMaxWarps)
+template <typename R, int M, bool PAIR, bool CORR, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
 k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in, Gm2dWork<R> wk,
              int rows, const SolveState *st, double *check) {
   constexpr int NQP = Gram<M>::NQP;
   using G = Strip<M>;
   using S = typename GramSum<R>::T;
-  __shared__ S sums[kMaxWarps * NQP];
+  __shared__ S sums[WARPS * NQP];
   const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const MarchWork work(L, rows, G::F, G::OW, M);
   griddep_wait();
@@ -405,6 +415,8 @@ k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in
     else basis_run<R, M, PAIR, UNIFORM, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
   }
   // block sums, in a fixed order
+#pragma unroll
+  for (int i = 0; i < NQP; ++i) acc[i].close();
   constexpr int SH = NQP == 16 ? 1 : 3;   // lane l holds quantity l >> SH
   const GramAcc<R, PAIR> v = gram_warp_sum<GramAcc<R, PAIR>, NQP>(acc);
   if ((lane & ((1 << SH) - 1)) == 0) sums[warp * NQP + (lane >> SH)] = gram_store(v);
@@ -475,8 +487,9 @@ __device__ __forceinline__ void update_run(const LevelK<R> &L, const Gm2dIn<R> &
       }
     }
   };
-  if (REST) m.run(y0 - 1, y1 + 2, w0, hook, emit);
-  else m.run(y0, y1, w0, hook, emit);
+  auto nofold = [] {};
+  if (REST) m.run(y0 - 1, y1 + 2, w0, hook, emit, nofold);
+  else m.run(y0, y1, w0, hook, emit, nofold);
 }
 
 template <typename R, int M, bool CORR, bool REST>
@@ -526,7 +539,7 @@ bool use_tiles(int N, int batch) {
 // about 12 warps per SM over the batch.  Blocks: about one per SM, so that few
 // partial sums reach the update kernel.
 template <> Gm2dPlan gm2d_plan<float>(int N, int m, int batch, int sms, bool restrict_) {
-  auto split = [&](int width, int cap, int *rows, int *warps, int *blocks) {
+  auto split = [&](int width, int cap, int wmax, int *rows, int *warps, int *blocks) {
     const int strips = (N + width - 1) / width;
     const long long want = 12LL * sms;
     long long r = ((long long)N * strips * batch + want - 1) / want;
@@ -534,15 +547,17 @@ template <> Gm2dPlan gm2d_plan<float>(int N, int m, int batch, int sms, bool res
     *rows = even_up((int)r);
     const int total = strips * ((N + *rows - 1) / *rows);
     const int most = total + total / 4;   // general runs are halved (MarchWork)
-    const int per = (int)std::min<long long>(kMaxWarps, std::max<long long>(1, ((long long)most * batch + sms - 1) / sms));
+    const int per = (int)std::min<long long>(wmax, std::max<long long>(1, ((long long)most * batch + sms - 1) / sms));
     *warps = per;
     *blocks = (most + per - 1) / per;
     if (cap > 0) *blocks = std::min(*blocks, cap);
   };
   Gm2dPlan p;
   p.tile = use_tiles(N, batch);
-  split(30 - 2 * m, gm2d_max_parts(batch, sms), &p.rows, &p.warps, &p.blocks);
-  split(restrict_ ? 28 - 2 * m : 32 - 2 * m, 0, &p.urows, &p.uwarps, &p.ublocks);
+  const int cap = gm2d_max_parts(batch, sms);
+  split(30 - 2 * m, cap, N > kGramPairMaxN ? kPlainWarps : kMaxWarps, &p.rows, &p.warps, &p.blocks);
+  if (N > kGramPairMaxN && p.blocks == cap) split(30 - 2 * m, cap, kMaxWarps, &p.rows, &p.warps, &p.blocks);
+  split(restrict_ ? 28 - 2 * m : 32 - 2 * m, 0, kMaxWarps, &p.urows, &p.uwarps, &p.ublocks);
   if (p.tile) {
     const int nt = (N + kBasisTile - 1) / kBasisTile;
     p.blocks = nt * nt;
@@ -565,10 +580,12 @@ void launch_gm2d_basis<float>(const LevelK<float> &L, float2 sigma, float s, int
                  p.rows, st, check);
     };
     const bool pair = L.N <= kGramPairMaxN;
-    if (pair && in.e) go(k_gm2d_basis<float, M, true, true>);
-    else if (pair) go(k_gm2d_basis<float, M, true, false>);
-    else if (in.e) go(k_gm2d_basis<float, M, false, true>);
-    else go(k_gm2d_basis<float, M, false, false>);
+    if (pair && in.e) go(k_gm2d_basis<float, M, true, true, kMaxWarps>);
+    else if (pair) go(k_gm2d_basis<float, M, true, false, kMaxWarps>);
+    else if (p.warps <= kPlainWarps && in.e) go(k_gm2d_basis<float, M, false, true, kPlainWarps>);
+    else if (p.warps <= kPlainWarps) go(k_gm2d_basis<float, M, false, false, kPlainWarps>);
+    else if (in.e) go(k_gm2d_basis<float, M, false, true, kMaxWarps>);
+    else go(k_gm2d_basis<float, M, false, false, kMaxWarps>);
   });
 }
 

@@ -245,7 +245,13 @@ k_gm3d_gram(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dWork<R> w
     if (M == 3) v[M - 1] = cfma(t, q1, cscale(cadd(ql, v[0]), R(0.5)));
     v[M] = cfma(t, ql, xl);
     gram_point<R, M, PAIR>(acc, v);
+    if (((z - W.z0) & 7) == 7) {
+#pragma unroll
+      for (int i = 0; i < Gram<M>::NQ; ++i) acc[i].fold();
+    }
   });
+#pragma unroll
+  for (int i = 0; i < Gram<M>::NQP; ++i) acc[i].close();
   store_gram<R, M, PAIR>(acc, wk, b, check);
 }
 
