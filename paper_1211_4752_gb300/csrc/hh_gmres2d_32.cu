@@ -346,10 +346,10 @@ struct MarchWork {
 };
 
 constexpr int kMaxWarps = 16;   // per block: 128 registers per thread
-// Plain sums, folded every four rows, need more: with 128 registers a 1023^2 step took
-// 57.2 us, with 168 and twelve warps 52.4 (four right-hand sides 146 and 138, 511^2 30.2 and
-// 29.2; unfolded, with 128 registers, 55.6, 139 and 29.4).  Where every warp has several
-// items 16 warps are faster all the same: 4095^2 483 us and 514 (unfolded 462).
+// Plain sums, folded every four rows, need more.  Twelve warps with 168 registers where
+// these hold all items at once (four right-hand sides at 511^2 38 us a step, 46 unfolded with
+// 128 registers; one at 1023^2 32.2 and 31.9), else 16 that spill a little (four at 1023^2 120
+// us and 126 with twelve, 113 unfolded; 4095^2 465 and 514, 443).
 constexpr int kPlainWarps = 12;
 
 template <typename R, int M, bool PAIR, int MODE, bool CORR>
@@ -544,9 +544,14 @@ template <> Gm2dPlan gm2d_plan<float>(int N, int m, int batch, int sms, bool res
     const long long want = 12LL * sms;
     long long r = ((long long)N * strips * batch + want - 1) / want;
     r = std::min<long long>(std::max<long long>(r, 4), 32);
-    *rows = even_up((int)r);
-    const int total = strips * ((N + *rows - 1) / *rows);
-    const int most = total + total / 4;   // general runs are halved (MarchWork)
+    int most;
+    // (longer where the items would not fit one block of wmax warps per SM: with a second
+    // wave of the 168-register blocks a 1023^2 step took 41 us)
+    for (*rows = even_up((int)r);; *rows += 2) {
+      const int total = strips * ((N + *rows - 1) / *rows);
+      most = total + total / 4;   // general runs are halved (MarchWork)
+      if (*rows >= 32 || (long long)most * batch <= (long long)wmax * sms) break;
+    }
     const int per = (int)std::min<long long>(wmax, std::max<long long>(1, ((long long)most * batch + sms - 1) / sms));
     *warps = per;
     *blocks = (most + per - 1) / per;
@@ -556,7 +561,7 @@ template <> Gm2dPlan gm2d_plan<float>(int N, int m, int batch, int sms, bool res
   p.tile = use_tiles(N, batch);
   const int cap = gm2d_max_parts(batch, sms);
   split(30 - 2 * m, cap, N > kGramPairMaxN ? kPlainWarps : kMaxWarps, &p.rows, &p.warps, &p.blocks);
-  if (N > kGramPairMaxN && p.blocks == cap) split(30 - 2 * m, cap, kMaxWarps, &p.rows, &p.warps, &p.blocks);
+  if (N > kGramPairMaxN && p.blocks * batch > sms) split(30 - 2 * m, cap, kMaxWarps, &p.rows, &p.warps, &p.blocks);
   split(restrict_ ? 28 - 2 * m : 32 - 2 * m, 0, kMaxWarps, &p.urows, &p.uwarps, &p.ublocks);
   if (p.tile) {
     const int nt = (N + kBasisTile - 1) / kBasisTile;
