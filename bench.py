@@ -457,12 +457,13 @@ def gmres_step_bytes(dim, kconst, mixed):
     """Algorithmic bytes per point of one GMRES(3) smoothing step on a level, each
     kernel reading and writing its vectors once.  2-D complex64: two kernels that read
     u, f (the basis is formed in both), u written: 40 B; complex128 stores the basis
-    instead: u, f in, q_0..q_2 out, u, q_0..q_2 in, u out: 160 B.  3-D: q_0, q_1 and q_2
-    by a kernel each, the Gram sums, the update: 128 or 256 B.  A k^2 field is read
-    once per kernel that forms products."""
+    instead: u, f in, q_0..q_2 and X q_2 out (96), those in for the coefficients (64), u,
+    q_0..q_2 in, u out (80): 240 B.  3-D: q_0, q_1 and q_2 by a kernel each, the Gram sums,
+    the update: 128 B; complex128 also stores X q_2 and reads all for the coefficients:
+    336 B.  A k^2 field is read once per kernel that forms products."""
     if dim == 2:
-        return (40.0 if mixed else 160.0) + (0.0 if kconst else 8.0)
-    return (128.0 + (0.0 if kconst else 16.0)) * (1.0 if mixed else 2.0)
+        return (40.0 if mixed else 240.0) + (0.0 if kconst else 8.0)
+    return 128.0 + (0.0 if kconst else 16.0) if mixed else 336.0 + (0.0 if kconst else 32.0)
 
 
 def gmres_record(w, args, k2_t, f, stream, flush):

@@ -1,5 +1,5 @@
 // GMRES(m) smoothing steps on 2-D levels with one reduction per step
-// (hh_gmres2d.cuhh; the method is described in hh_cheb.cuh).
+// (hh_gmres2d.cuh; the method is described in hh_cheb.cuh).
 #pragma once
 #include "hh_internal.h"
 #include "hh_cheb.cuh"

@@ -176,41 +176,39 @@ size_t tile_smem(int m, int ty) {
 
 // Basis of a tile whose iterate is in A and right-hand side in F: q_0 -> B,
 // q_1 -> A, q_2 -> F (M - 1 products), each with the block's barrier after it.
-// The region of q_j is the tile and M - j points (REST: one more, and one more
-// again at the high ends) around it.
-template <typename R, int M, int MODE, int TX, int XH, typename Sync>
+// The region of q_j is the tile and M - j points around it.
+template <typename R, int M, int MODE, int TX, int XH>
 __device__ __forceinline__ void tile_vectors(const TileCtx<R, MODE> &t, ColumnOp<R, MODE> &op, int H,
                                              typename Cx<R>::T *A, typename Cx<R>::T *B,
-                                             typename Cx<R>::T *F, int last, Sync sync) {
+                                             typename Cx<R>::T *F) {
   using C = typename Cx<R>::T;
   // q_0 on buffer [1, TX + XH - 1) x [1, H - 1)
   t.template walk<TX + XH - 2, true>(op, A, 1, H - 2, [&](int p, int, int) { return F[p]; },
                                      [&](int p, int, int, C r) { B[p] = r; });
-  sync();
-  if (M >= 2 && last >= 1) {
+  __syncthreads();
+  if (M >= 2) {
     t.template walk<TX + XH - 4, false>(op, B, 2, H - 4, [](int, int, int) { return C(); },
                                         [&](int p, int, int, C r) { A[p] = r; });
-    sync();
+    __syncthreads();
   }
-  if (M >= 3 && last >= 2) {
+  if (M >= 3) {
     t.template walk<TX + XH - 6, false>(op, A, 3, H - 6, [](int, int, int) { return C(); },
                                         [&](int p, int, int, C r) { F[p] = cmk(fmaf_any(R(2), r.x, -B[p].x), fmaf_any(R(2), r.y, -B[p].y)); });
-    sync();
+    __syncthreads();
   }
 }
 
-template <typename R, int M, bool PAIR, int MODE, bool CORR>
+template <typename R, int M, int MODE, bool CORR>
 __device__ __forceinline__ void basis_body(const LevelK<R> &L, const Gm2dWork<R> &wk,
                                            typename Cx<R>::T sigma, R s, int b, int bx, int by,
                                            int ty, typename Cx<R>::T *A, typename Cx<R>::T *B,
                                            typename Cx<R>::T *F, const typename Cx<R>::T *sr,
-                                           GramAcc<R, PAIR> (&acc)[Gram<M>::NQP]) {
+                                           GramAcc<R, false> (&acc)[Gram<M>::NQP]) {
   using C = typename Cx<R>::T;
-  constexpr bool STORE = sizeof(R) == 8;
   constexpr int XH = 2 * (M + 1);
   const TileCtx<R, MODE> t{L, bx, by, sr};
   ColumnOp<R, MODE> op(L, sigma, s);
-  tile_vectors<R, M, MODE, kTX, XH>(t, op, ty + XH, A, B, F, M - 1, [] { __syncthreads(); });
+  tile_vectors<R, M, MODE, kTX, XH>(t, op, ty + XH, A, B, F);
   const C sg = cscale(sigma, s);
   const C *src = M == 1 ? B : (M == 2 ? A : F);
   t.template walk<kTX, false>(op, src, M + 1, ty, [](int, int, int) { return C(); },
@@ -229,8 +227,8 @@ __device__ __forceinline__ void basis_body(const LevelK<R> &L, const Gm2dWork<R>
       v[M - 1] = shifted(A[p], cscale(cadd(F[p], v[0]), R(0.5)));
       v[M] = shifted(F[p], xl);
     }
-    gram_point<R, M, PAIR>(acc, v);
-    if (STORE && x < L.N && y < L.N) {
+    gram_point<R, M, false>(acc, v);
+    if (x < L.N && y < L.N) {
       C *q = wk.q + (size_t)b * L.S + (size_t)y * L.P + x;
       q[0] = v[0];
       if (M >= 2) q[wk.qs] = A[p];
@@ -247,7 +245,6 @@ k_gm2d_basis(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<doubl
              int ty, const SolveState *st, double *check) {
   using R = double;
   using C = double2;
-  constexpr bool PAIR = false;
   constexpr int NQP = Gram<M>::NQP, NW = kTileThreads / 32;
   using S = typename GramSum<R>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -261,7 +258,8 @@ k_gm2d_basis(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<doubl
   const bool zero = __syncthreads_or(in.zero_mode == ZERO_ALL ||
                                      (in.zero_mode == ZERO_FLAG && st && st[b].zero)) != 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) wk.zflag[b] = zero;
-  GramAcc<R, PAIR> acc[NQP];
+  using Acc = GramAcc<R, false>;
+  Acc acc[NQP];
 #pragma unroll
   for (int i = 0; i < NQP; ++i) acc[i].zero();
   const int N = L.N, nx = (N + kTX - 1) / kTX, ntiles = nx * ((N + ty - 1) / ty);
@@ -271,17 +269,17 @@ k_gm2d_basis(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<doubl
     if (i != (int)blockIdx.x) __syncthreads();   // the previous tile's last reads
     stage_tile<R, CORR>(L, in, b, zero, mode == GENERAL, bx, by, ty + 2 * (M + 1), A, F, sr);
     __syncthreads();
-    if (mode == UNIFORM_K) basis_body<R, M, PAIR, UNIFORM_K, CORR>(L, wk, sigma, s, b, bx, by, ty, A, B, F, sr, acc);
-    else if (mode == UNIFORM) basis_body<R, M, PAIR, UNIFORM, CORR>(L, wk, sigma, s, b, bx, by, ty, A, B, F, sr, acc);
-    else basis_body<R, M, PAIR, GENERAL, CORR>(L, wk, sigma, s, b, bx, by, ty, A, B, F, sr, acc);
+    if (mode == UNIFORM_K) basis_body<R, M, UNIFORM_K, CORR>(L, wk, sigma, s, b, bx, by, ty, A, B, F, sr, acc);
+    else if (mode == UNIFORM) basis_body<R, M, UNIFORM, CORR>(L, wk, sigma, s, b, bx, by, ty, A, B, F, sr, acc);
+    else basis_body<R, M, GENERAL, CORR>(L, wk, sigma, s, b, bx, by, ty, A, B, F, sr, acc);
   }
   // block sums, in a fixed order
   constexpr int SH = NQP == 16 ? 1 : 3;   // lane l holds quantity l >> SH
-  const GramAcc<R, PAIR> v = gram_warp_sum<GramAcc<R, PAIR>, NQP>(acc);
+  const Acc v = gram_warp_sum<Acc, NQP>(acc);
   if ((lane & ((1 << SH) - 1)) == 0) sums[warp * NQP + (lane >> SH)] = gram_store(v);
   __syncthreads();
   if (threadIdx.x < NQP) {
-    GramAcc<R, PAIR> t;
+    Acc t;
     t.zero();
     for (int i = 0; i < NW; ++i) gram_add(t, sums[i * NQP + threadIdx.x]);
     const S g = gram_store(t);

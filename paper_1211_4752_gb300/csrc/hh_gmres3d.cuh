@@ -50,7 +50,7 @@ template <typename R> struct Walk3 {
   }
 };
 
-// A of one column; UNI: coefficients uniform and real on the block's points.
+// A of one column.
 template <typename R> struct Column3 {
   using C = typename Cx<R>::T;
   C lx, ux, ly, uy, d;     // d: diagonal without its z part (less beta k^2 where k is constant)
