@@ -25,10 +25,11 @@
 // of FP32 values (Dekker / Knuth: the product's and the sum's rounding errors are kept in a
 // second FP32 value), which costs no FP64 arithmetic.  On levels of more than
 // kGramPairMaxN points per axis a thread's own sums are plain FP32, folded into a second
-// value every four rows (3-D: eight planes), and pairs from there on: relative errors of
-// 2.7e-10 (511^2), 2.3e-10 (1023^2), 1.3e-10 (2047^2), 6.1e-10 (511^2, 16 right-hand
-// sides) and 1.9e-10 (127^3; 3.6e-10 with 16); without the folds up to 1.3e-9 and 2.5e-9, with FP32
-// warp sums added in FP64 4.4e-10 to 7.2e-10.  What the nearly parallel vectors of a smooth
+// value every four rows (3-D: eight planes; above 1024 points per axis after each run of
+// rows), and pairs from there on: relative errors of 2.7e-10 (511^2), 2.3e-10 (1023^2),
+// 4.0e-10 (2047^2), 6.1e-10 (511^2, 16 right-hand sides) and 1.9e-10 (127^3; 3.6e-10 with
+// 16); without the folds up to 1.3e-9 and 2.5e-9, with FP32 warp sums added in FP64 4.4e-10
+// to 7.2e-10.  What the nearly parallel vectors of a smooth
 // residual lose to their own rounding stays: a complex64 cycle from zero on smooth
 // right-hand sides is 1 to 5 times as far from the exact one as with an orthogonalised
 // basis (the step's residual is the same to 1e-7), on rough ones no further.

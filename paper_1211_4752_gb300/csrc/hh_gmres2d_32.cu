@@ -349,10 +349,15 @@ constexpr int kMaxWarps = 16;   // per block: 128 registers per thread
 // Plain sums, folded every four rows, need more.  Twelve warps with 168 registers where
 // these hold all items at once (four right-hand sides at 511^2 38 us a step, 46 unfolded with
 // 128 registers; one at 1023^2 32.2 and 31.9), else 16 that spill a little (four at 1023^2 120
-// us and 126 with twelve, 113 unfolded; 4095^2 465 and 514, 443).
+// us and 126 with twelve, 113 unfolded).
 constexpr int kPlainWarps = 12;
+// Larger levels have so many runs that a warp's sums of whole ones are near enough (4.0e-10
+// at 2047^2, 5.2e-10 with FP32 warp sums added in FP64): added up as pairs after each item,
+// 2047^2 112 us a step, 4095^2 441 (folded every four rows 119 and 458, not at all 110 and 436).
+constexpr int kFoldRowsMaxN = 1024;
+enum { PAIRED, FOLD_ROWS, FOLD_ITEM };
 
-template <typename R, int M, bool PAIR, int MODE, bool CORR>
+template <typename R, int M, bool PAIR, int SUMS, int MODE, bool CORR>
 __device__ __forceinline__ void basis_run(const LevelK<R> &L, const Gm2dIn<R> &in,
                                           typename Cx<R>::T sigma, R s, R g, int b, bool zero, int x,
                                           int y0, int y1, bool own,
@@ -376,12 +381,13 @@ __device__ __forceinline__ void basis_run(const LevelK<R> &L, const Gm2dIn<R> &i
     gram_point<R, M, PAIR>(acc, v);
   };
   m.run(y0, y1, none0, none, emit, [&] {
+    if (SUMS != FOLD_ROWS) return;
 #pragma unroll
     for (int i = 0; i < Gram<M>::NQ; ++i) acc[i].fold();
   });
 }
 
-template <typename R, int M, bool PAIR, bool CORR, int WARPS>
+template <typename R, int M, bool PAIR, bool CORR, int WARPS, int SUMS>
 __global__ void __launch_bounds__(32 * WARPS)
 k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in, Gm2dWork<R> wk,
              int rows, const SolveState *st, double *check) {
@@ -401,25 +407,43 @@ k_gm2d_basis(LevelK<R> L, typename Cx<R>::T sigma, R s, int kconst, Gm2dIn<R> in
     wk.zflag[b] = zero;
     wk.g[b] = g;
   }
+  constexpr int SH = NQP == 16 ? 1 : 3;   // lane l holds quantity l >> SH of a warp's sums
+  const bool holds = (lane & ((1 << SH) - 1)) == 0;
+  S *mine = sums + warp * NQP + (lane >> SH);
   GramAcc<R, PAIR> acc[NQP];
+  auto clear = [&] {
 #pragma unroll
-  for (int i = 0; i < NQP; ++i) acc[i].zero();
+    for (int i = 0; i < NQP; ++i) acc[i].zero();
+  };
+  clear();
+  if (SUMS == FOLD_ITEM && holds) *mine = make_float2(0.f, 0.f);
   const bool own = lane >= G::F && lane < G::F + G::OW;
   for (int wi = blockIdx.x * nw + warp; wi < work.items(); wi += gridDim.x * nw) {
     int strip, y0, y1;
     const bool uni = work.item(wi, L.N, strip, y0, y1);
     const int x = strip * G::OW - G::F + lane;
     if (y0 >= y1) continue;
-    if (!uni) basis_run<R, M, PAIR, GENERAL, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
-    else if (kconst) basis_run<R, M, PAIR, UNIFORM_K, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
-    else basis_run<R, M, PAIR, UNIFORM, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
+    if (!uni) basis_run<R, M, PAIR, SUMS, GENERAL, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
+    else if (kconst) basis_run<R, M, PAIR, SUMS, UNIFORM_K, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
+    else basis_run<R, M, PAIR, SUMS, UNIFORM, CORR>(L, in, sigma, s, g, b, zero, x, y0, y1, own, acc);
+    if (SUMS == FOLD_ITEM) {
+      GramAcc<R, PAIR> v = gram_warp_sum<GramAcc<R, PAIR>, NQP>(acc);
+      if (holds) {
+        gram_add(v, *mine);
+        *mine = gram_store(v);
+      }
+      clear();
+    }
   }
   // block sums, in a fixed order
+  if (SUMS != FOLD_ITEM) {
+    if (SUMS == FOLD_ROWS) {
 #pragma unroll
-  for (int i = 0; i < NQP; ++i) acc[i].close();
-  constexpr int SH = NQP == 16 ? 1 : 3;   // lane l holds quantity l >> SH
-  const GramAcc<R, PAIR> v = gram_warp_sum<GramAcc<R, PAIR>, NQP>(acc);
-  if ((lane & ((1 << SH) - 1)) == 0) sums[warp * NQP + (lane >> SH)] = gram_store(v);
+      for (int i = 0; i < NQP; ++i) acc[i].close();
+    }
+    const GramAcc<R, PAIR> v = gram_warp_sum<GramAcc<R, PAIR>, NQP>(acc);
+    if (holds) *mine = gram_store(v);
+  }
   __syncthreads();
   if (threadIdx.x < NQP) {
     GramAcc<R, PAIR> t;
@@ -584,13 +608,15 @@ void launch_gm2d_basis<float>(const LevelK<float> &L, float2 sigma, float s, int
       launch_pdl(k, dim3(p.blocks, batch), dim3(32 * p.warps), 0, stream, L, sigma, s, kconst, in, w,
                  p.rows, st, check);
     };
-    const bool pair = L.N <= kGramPairMaxN;
-    if (pair && in.e) go(k_gm2d_basis<float, M, true, true, kMaxWarps>);
-    else if (pair) go(k_gm2d_basis<float, M, true, false, kMaxWarps>);
-    else if (p.warps <= kPlainWarps && in.e) go(k_gm2d_basis<float, M, false, true, kPlainWarps>);
-    else if (p.warps <= kPlainWarps) go(k_gm2d_basis<float, M, false, false, kPlainWarps>);
-    else if (in.e) go(k_gm2d_basis<float, M, false, true, kMaxWarps>);
-    else go(k_gm2d_basis<float, M, false, false, kMaxWarps>);
+    auto corr = [&](auto c) {
+      constexpr bool CORR = decltype(c)::value;
+      if (L.N <= kGramPairMaxN) go(k_gm2d_basis<float, M, true, CORR, kMaxWarps, PAIRED>);
+      else if (p.warps <= kPlainWarps) go(k_gm2d_basis<float, M, false, CORR, kPlainWarps, FOLD_ROWS>);
+      else if (L.N <= kFoldRowsMaxN) go(k_gm2d_basis<float, M, false, CORR, kMaxWarps, FOLD_ROWS>);
+      else go(k_gm2d_basis<float, M, false, CORR, kMaxWarps, FOLD_ITEM>);
+    };
+    if (in.e) corr(std::true_type());
+    else corr(std::false_type());
   });
 }
 
