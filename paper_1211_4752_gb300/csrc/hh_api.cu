@@ -1758,11 +1758,10 @@ hh_status autotune(hh_handle *h, cudaStream_t s) {
 // memory (HH_GMTAIL=off in the environment keeps every level per-level).
 // Largest level (points per axis) of the GMRES one-block tail (HH_GMTAIL_N
 // overrides, for tuning).  A step of the many-block kernels takes 5 to 6 us on any
-// small level (complex64; 3-D 8 to 9), one of the tail about 4 us on 15^2, but the
-// tail's one SM falls behind as the points grow: the 1023^2 cycle takes 210.9 us
-// with the tail from 15^2 and 212.8 from 31^2 (255^2: 129 from 63^2, 100 from 31^2,
-// 98 from 15^2, 102 from 7^2), the 127^3 cycle 335 us from 7^3 and 393 from 15^3; in
-// complex128 (255^2, four right-hand sides) 0.73 ms from 15^2 and 0.78 from 31^2.
+// small level (complex64; 3-D 8 to 10), one of the tail about 4 us on 15^2, but the
+// tail's one SM falls behind as the points grow: the 1023^2 cycle takes 215 us with
+// the tail from 7^2, 208 from 15^2 and 209 from 31^2 (255^2: 96, 90, 90), the 127^3
+// cycle 336 us from 7^3 and 373 from 15^3; in complex128 (255^2) 525 us, 524 and 612.
 int gm_tail_max_n(int dim) {
   if (const char *e = std::getenv("HH_GMTAIL_N")) return std::max(3, std::atoi(e));
   return dim == 3 ? 7 : 15;

@@ -171,7 +171,7 @@ __device__ __forceinline__ C resid_uniform(C fv, C vc, C sn, C c0, C Dk) {
 // complex128, whose kernels are bound by the FP64 pipe.  Measured with the weight made
 // on the host (LevelK::wk) and three blocks per SM: a 1023^2 down pass 143 -> 115-121 us,
 // up pass 87 -> 74, 511^2 50 -> 44 and 35 -> 24; per point about 50 and 35 FP64
-// instructions, which at the pipe's 64 cycles per warp take 85 to 90 % of the time.
+// instructions; the pipe, 64 cycles per warp and instruction, is 86 and 85 % busy.
 template <typename C, typename R>
 __device__ __forceinline__ void jacobi_real(C fv, C uc, C sn, R c0, R dk, R wk, C &r, C &v) {
   r.x = fmaf_any(-dk, uc.x, fmaf_any(c0, sn.x, fv.x));

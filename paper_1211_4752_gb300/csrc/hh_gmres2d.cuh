@@ -111,12 +111,40 @@ __device__ __forceinline__ void step_coef(const typename GramSum<R>::T *parts, i
 }
 
 // complex128: the coefficients that k_gm2d_coef stored, with the correction from its nb
-// blocks' sums.  One warp; sums: 8 slots.
+// blocks' sums.  By the whole block (sums: 8 slots per warp), ends with its barrier: one
+// warp waits for ten rounds of loads at 152 blocks.
+template <int M>
+__device__ __forceinline__ void read_coef_block(const Gm2dWork<double> &wk, int b, int nb, double s,
+                                                double *sums, StepCoef<double> *out) {
+  const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
+  static_assert(sizeof(StepCoef<double>) == kGm2dCoef * sizeof(double), "coefficients");
+  if (tid < kGm2dCoef) reinterpret_cast<double *>(out)[tid] = wk.coef[(size_t)b * kGm2dCoef + tid];
+  const double *p = wk.parts2 + (size_t)b * kGm2dCorr * 8 + (tid & 7);
+  double d = 0.0;
+#pragma unroll 4
+  for (int i = tid >> 3; i < nb; i += 4 * nw) d += p[(size_t)i * 8];
+  d += __shfl_xor_sync(0xffffffffu, d, 8);
+  d += __shfl_xor_sync(0xffffffffu, d, 16);
+  if (lane < 8) sums[(tid >> 5) * 8 + lane] = d;
+  __syncthreads();
+  if (tid < 32) {
+    d = 0.0;
+    for (int w = lane >> 3; w < nw; w += 4) d += sums[w * 8 + (lane & 7)];
+    d += __shfl_xor_sync(0xffffffffu, d, 8);
+    d += __shfl_xor_sync(0xffffffffu, d, 16);
+    __syncwarp();
+    if (lane < 8) sums[lane] = d;
+    __syncwarp();
+    solve_correction<M>(sums, s, out);
+  }
+  __syncthreads();
+}
+// The same by one warp (the tiles, whose other warps form the basis meanwhile); sums: 8
+// slots.
 template <int M>
 __device__ __forceinline__ void read_coef(const Gm2dWork<double> &wk, int b, int nb, double s,
                                           double *sums, StepCoef<double> *out) {
   const int lane = threadIdx.x & 31;
-  static_assert(sizeof(StepCoef<double>) == kGm2dCoef * sizeof(double), "coefficients");
   if (lane < kGm2dCoef) reinterpret_cast<double *>(out)[lane] = wk.coef[(size_t)b * kGm2dCoef + lane];
   const double *p = wk.parts2 + (size_t)b * kGm2dCorr * 8 + (lane & 7);
   double t[4] = {0.0, 0.0, 0.0, 0.0};

@@ -14,13 +14,13 @@
 // per tile, a thread per point (hh_gmres2d.cuh), because there one warp's chain
 // of march iterations is the time.
 //
-// Measured (GB300, one right-hand side, constant k with layers): a GMRES(3) step
-// takes 31.8 us at 1023^2 (67.6 with a kernel and a reduction per Arnoldi step),
-// 18.2 at 511^2 (41.7), 12.0 at 255^2 (36.4), 6.7 at 127^2 (30.3) and 6.2 at 63^2
-// (29.3; 20.6 with marches); the 1023^2 cycle 217 us (541).  At 1023^2 the two
-// kernels issue 10 instructions per point and warp at half the issue rate; two
-// columns per lane, or the tiles of hh_gmres2d_64.cu, were slower (44 and 54 us
-// a step).
+// Measured (GB300, one right-hand side, constant k with layers; in brackets a kernel and a
+// reduction per Arnoldi step): a GMRES(3) step takes 32.1 us at 1023^2 (67.2), 18.6 at 511^2
+// (41.6), 10.9 at 255^2 (36.4), 6.8 at 127^2 (30.3) and 6.3 at 63^2 (29.5; 20.6 with
+// marches); the 1023^2 cycle 207 us (539).  At 1023^2 the basis kernel uses 45 % and the
+// update 41 % of the issue slots with 12 and 15 warps per SM: chains of dependent rows; at
+// 2047^2 59 and 46 %.  Two columns per lane, or the tiles of hh_gmres2d_64.cu, were slower
+// (44 and 54 us a step).
 #include "hh_gmres2d.cuh"
 
 namespace hh {

@@ -5,11 +5,13 @@
 // small: a block works on tiles of 56 columns and up to 32 rows in shared memory,
 // a thread per column and run of rows, the values above and below carried in
 // registers.  Small levels: a thread per point of 8 x 8 tiles (hh_gmres2d.cuh).
-// Measured (GB300; in brackets a kernel and a reduction per Arnoldi step): a GMRES(3)
-// step takes 412 us at 1023^2 (393; with marches 669), 139 at 511^2 (139), 59 at
-// 255^2 (75), 40 at 127^2 (50) and 21 at 63^2 (48), and of four right-hand sides at
-// 1023^2 1204 (1420); the cycle of one at 1023^2 1.71 ms (1.98), of four there 4.58
-// (5.49) and at 255^2 0.71 (1.05).
+// Measured (GB300, constant k with layers; in brackets a kernel and a reduction per Arnoldi
+// step): a GMRES(3) step takes 479 us at 1023^2 (394), 165 at 511^2 (140), 90 at 255^2 (76),
+// 38 at 127^2 (51) and 24 at 63^2 (51), and of four right-hand sides at 1023^2 1460 (1424);
+// the cycle of one at 1023^2 1.98 ms (1.99), of four there 5.40 (5.49) and at 255^2 0.82
+// (1.05).  A fifth of a step is the correction of its coefficients (k_gm2d_coef), without
+// which these kernels lose digits.  The FP64 pipe is 86 % busy in the basis kernel at 1023^2,
+// 92 % in k_gm2d_coef and 71 to 76 % in the update.
 #include "hh_gmres2d.cuh"
 #include "hh_gmres3d.h"
 
@@ -25,8 +27,9 @@ template <typename R, int MODE> struct ColumnOp {
   C c0, D0, sb, sd;        // uniform: c_0, 4 c_0, s beta, s (4 c_0 - sigma)
   C lo, up, dg, dgs, sigma, beta;   // dgs = dg - sigma
   R cf, s, kc;
+  bool realb;              // beta is real (a comparison per point is an FP64 instruction)
   __device__ __forceinline__ ColumnOp(const LevelK<R> &L, C sigma_, R s_)
-      : sigma(sigma_), beta(L.beta), s(s_), kc(L.kc) {
+      : sigma(sigma_), beta(L.beta), s(s_), kc(L.kc), realb(L.beta.y == R(0)) {
     if (MODE != GENERAL) {
       c0 = L.c0;
       D0 = cscale(c0, R(4));
@@ -62,7 +65,7 @@ template <typename R, int MODE> struct ColumnOp {
       // the products with zero here and below)
       const R dx = fmaf_any(-sb.x, kv, sd.x);
       r = cmk(fmaf_any(dx, v.x, r.x), fmaf_any(dx, v.y, r.y));
-      if (beta.y != R(0)) {
+      if (!realb) {
         const R dy = fmaf_any(-sb.y, kv, sd.y);
         r = cmk(fmaf_any(-dy, v.y, r.x), fmaf_any(dy, v.x, r.y));
       }
@@ -80,7 +83,7 @@ template <typename R, int MODE> struct ColumnOp {
     C r;
     r.x = fmaf_any(c0.x, sn.x, fmaf_any(-dx, v.x, f.x));
     r.y = fmaf_any(c0.x, sn.y, fmaf_any(-dx, v.y, f.y));
-    if (beta.y != R(0)) {
+    if (!realb) {
       const R dy = beta.y * kk;
       r = cmk(fmaf_any(-dy, v.y, r.x), fmaf_any(dy, v.x, r.y));
     }
@@ -210,6 +213,7 @@ __device__ __forceinline__ void basis_body(const LevelK<R> &L, const Gm2dWork<R>
   ColumnOp<R, MODE> op(L, sigma, s);
   tile_vectors<R, M, MODE, kTX, XH>(t, op, ty + XH, A, B, F);
   const C sg = cscale(sigma, s);
+  const bool reals = sg.y == R(0);
   const C *src = M == 1 ? B : (M == 2 ? A : F);
   t.template walk<kTX, false>(op, src, M + 1, ty, [](int, int, int) { return C(); },
                               [&](int p, int x, int y, C xl) {
@@ -217,7 +221,7 @@ __device__ __forceinline__ void basis_body(const LevelK<R> &L, const Gm2dWork<R>
     v[0] = B[p];
     auto shifted = [&](C q, C xq) {   // X q + s sigma q
       C r = cmk(fmaf_any(sg.x, q.x, xq.x), fmaf_any(sg.x, q.y, xq.y));
-      if (sg.y != R(0)) r = cmk(fmaf_any(-sg.y, q.y, r.x), fmaf_any(sg.y, q.x, r.y));
+      if (!reals) r = cmk(fmaf_any(-sg.y, q.y, r.x), fmaf_any(sg.y, q.x, r.y));
       return r;
     };
     if (M == 1) v[1] = shifted(v[0], xl);
@@ -316,7 +320,8 @@ __device__ __forceinline__ void restrict_body(const TileCtx<R, MODE> &t, ColumnO
 // The step's coefficients from the partial Gram matrices, for the update kernel
 // (every block of this kernel adds and solves; block 0 stores), and per block the sums of
 // their correction (solve_correction) from the stored vectors.  Bound by the FP64 pipe
-// (about 32 instructions per point): 88 us at 1023^2, 39 at 511^2, 11 on small levels.
+// (92 % busy, 32 instructions per point on the finest level, 38 below): 77 us at 1023^2, 40
+// at 511^2, 11 on small levels.
 template <int M>
 __global__ void __launch_bounds__(1024)
 k_gm2d_coef(LevelK<double> L, int rows, double2 sigma, double s, Gm2dWork<double> wk, int nparts,
@@ -339,26 +344,32 @@ k_gm2d_coef(LevelK<double> L, int rows, double2 sigma, double s, Gm2dWork<double
 #pragma unroll
   for (int j = 0; j < M; ++j) y[j] = cscale(sc.z[j], (M == 3 && j == 1 ? 0.5 : 1.0) / s);
   const double2 t = cscale(sigma, s), t2 = cadd(t, t);
-  auto shifted = [](double2 c, double2 q, double2 xq) {   // xq + c q (c: real on the finest level)
-    double2 r = make_double2(fma(c.x, q.x, xq.x), fma(c.x, q.y, xq.y));
-    if (c.y != 0.0) r = make_double2(fma(-c.y, q.y, r.x), fma(c.y, q.x, r.y));
-    return r;
-  };
   const double2 *q = wk.q + (size_t)b * L.S;
   const int N = L.N;
-  for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < (unsigned)rows * (unsigned)N; p += gridDim.x * blockDim.x) {
-    const unsigned yy = p / (unsigned)N, o = yy * (unsigned)L.P + (p - yy * (unsigned)N);
-    double2 v[M + 1], a[M];
+  // (real t, the finest level's: two loops; with a condition in one both sides' products
+  // were formed, 89 us)
+  auto walk = [&](auto real) {
+    auto shifted = [](double2 c, double2 q, double2 xq) {   // xq + c q
+      double2 r = make_double2(fma(c.x, q.x, xq.x), fma(c.x, q.y, xq.y));
+      if (!decltype(real)::value) r = make_double2(fma(-c.y, q.y, r.x), fma(c.y, q.x, r.y));
+      return r;
+    };
+    for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < (unsigned)rows * (unsigned)N; p += gridDim.x * blockDim.x) {
+      const unsigned yy = p / (unsigned)N, o = yy * (unsigned)L.P + (p - yy * (unsigned)N);
+      double2 v[M + 1], a[M];
 #pragma unroll
-    for (int j = 0; j <= M; ++j) v[j] = q[(size_t)j * wk.qs + o];   // v[M] = X q_{M-1}
-    a[0] = shifted(t, v[0], v[1]);
-    if (M == 2) a[M - 1] = shifted(t, v[1], v[M]);
-    if (M == 3) {   // (twice a_1, with half of y_1 and of d_1)
-      a[1 % M] = shifted(t2, v[1], cadd(v[2 % (M + 1)], v[0]));
-      a[M - 1] = shifted(t, v[M - 1], v[M]);
+      for (int j = 0; j <= M; ++j) v[j] = q[(size_t)j * wk.qs + o];   // v[M] = X q_{M-1}
+      a[0] = shifted(t, v[0], v[1]);
+      if (M == 2) a[M - 1] = shifted(t, v[1], v[M]);
+      if (M == 3) {   // (twice a_1, with half of y_1 and of d_1)
+        a[1 % M] = shifted(t2, v[1], cadd(v[2 % (M + 1)], v[0]));
+        a[M - 1] = shifted(t, v[M - 1], v[M]);
+      }
+      correction_point<M>(acc, a, y, v[0]);
     }
-    correction_point<M>(acc, a, y, v[0]);
-  }
+  };
+  if (t.y == 0.0) walk(std::true_type());
+  else walk(std::false_type());
   const A v = gram_warp_sum<A, 8>(acc);
   __syncthreads();   // (block 0 has read the coefficients; the Gram sums are used up)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -381,7 +392,7 @@ k_gm2d_update(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<doub
                      double2 *fc, double2 cs, Lay lc, const SolveState *st) {
   constexpr int TX = kTX, O = REST ? 1 : 0, XH = REST ? 3 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double sums[8];
+  __shared__ double sums[kTileThreads / 4];
   __shared__ StepCoef<double> sc;
   const int hb = tile_rows(M, ty);
   double2 *A = reinterpret_cast<double2 *>(smem_raw), *B = A + hb * kTP, *sr = B + 2 * hb * kTP;
@@ -390,8 +401,7 @@ k_gm2d_update(LevelK<double> L, double2 sigma, double s, int kconst, Gm2dIn<doub
   griddep_launch_dependents();
   if (!__syncthreads_and(!(st && !st[b].active))) return;
   const bool zero = wk.zflag[b] != 0;
-  if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, sums, &sc);
-  __syncthreads();
+  read_coef_block<M>(wk, b, nparts, s, sums, &sc);
   const double2 *q = wk.q + (size_t)b * L.S;
   u_out += (size_t)b * L.S;
   if (REST) fc += (size_t)b * lc.S;

@@ -10,9 +10,9 @@
 // carried in registers, the four lateral ones come from L1, and the coefficients of
 // x and y stay in registers.
 //
-// Measured (GB300, complex64, GMRES(3)): a step takes 78 us at 127^3 (152 with a
-// reduction per Arnoldi step), 23 at 63^3 (49) and 9.6 at 31^3 (34); the 127^3 cycle
-// 335 us (650).  complex128, 63^3: 129 us (152).
+// Measured (GB300, complex64, GMRES(3)): a step takes 76 us at 127^3 (151 with a
+// reduction per Arnoldi step), 23 at 63^3 (49) and 10.4 at 31^3 (34); the 127^3 cycle
+// 336 us (674).  complex128, 63^3: 154 us (154), the cycle 642 (734).
 #pragma once
 #include "hh_kernels.cuh"
 #include "hh_launch.cuh"
@@ -273,8 +273,7 @@ k_gm3d_update(LevelK<R> L, R s, const typename Cx<R>::T *u_in, Gm2dWork<R> wk, i
     step_coef<R, M>(wk.parts + (size_t)b * nparts * NQP, nparts, s * gram_rcp(g), tol, sums, &sc);
     if (wk.track && blockIdx.x == 0 && threadIdx.x == 0) gram_estimate(wk.mag, b, sums[0], g);
   } else {
-    if (threadIdx.x < 32) read_coef<M>(wk, b, nparts, s, sums, &sc);
-    __syncthreads();
+    read_coef_block<M>(wk, b, nparts, s, sums, &sc);
   }
   C z[M];
 #pragma unroll

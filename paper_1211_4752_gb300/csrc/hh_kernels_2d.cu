@@ -15,7 +15,7 @@
 // Measured (GB300, complex128, 1023^2, variable k, three right-hand sides; before:
 // a thread per point, five reads, the general coefficients everywhere): operator
 // 143 -> 125 us, sweep 329 -> 246, residual + weighting 400 -> 225, correction +
-// sweep 633 -> 305; 85 to 90 % of each is the FP64 pipe (a warp's instruction takes
+// sweep 633 -> 305; 77 (operator) to 85 % of each is the FP64 pipe (a warp's instruction takes
 // 64 cycles).  Runs of 32 rows, one warp each, took 161 / 327 / 258 / 348: blocks of
 // general strips (layers) cost twice the others' work and set a single wave's time.
 // A sequence of operator, adjoint operator, sweep, restriction, correction and coarse
