@@ -11,7 +11,7 @@
 // the cycle of one at 1023^2 1.98 ms (1.99), of four there 5.40 (5.49) and at 255^2 0.82
 // (1.05).  A fifth of a step is the correction of its coefficients (k_gm2d_coef), without
 // which these kernels lose digits.  The FP64 pipe is 86 % busy in the basis kernel at 1023^2,
-// 92 % in k_gm2d_coef and 71 to 76 % in the update.
+// 89 % in k_gm2d_coef and 71 to 76 % in the update.
 #include "hh_gmres2d.cuh"
 #include "hh_gmres3d.h"
 
@@ -320,7 +320,7 @@ __device__ __forceinline__ void restrict_body(const TileCtx<R, MODE> &t, ColumnO
 // The step's coefficients from the partial Gram matrices, for the update kernel
 // (every block of this kernel adds and solves; block 0 stores), and per block the sums of
 // their correction (solve_correction) from the stored vectors.  Bound by the FP64 pipe
-// (92 % busy, 32 instructions per point on the finest level, 38 below): 77 us at 1023^2, 40
+// (89 % busy, 32 instructions per point on the finest level, 38 below): 77 us at 1023^2, 40
 // at 511^2, 11 on small levels.
 template <int M>
 __global__ void __launch_bounds__(1024)
